@@ -466,11 +466,11 @@ def run(s):
             _batch(s, max(0, len(frames) - 8), len(frames))
         out = s["out"]
         pos, keys, cube = maps[0].mesh(changed_only=case["changed"], cap=len(out["pos"]))
-        # triangles come in no fixed order: sorted by their cube
-        c = cube.long()
-        order = torch.sort(((c[:, 2] << 40) + (c[:, 1] << 20)) + c[:, 0], stable=True)[1]
-        for name, v in (("pos", pos), ("keys", keys), ("cube", cube)):
-            torch.index_select(v, 0, order, out=out[name][:len(order)])
+        # triangles come in no fixed order: sorted by their cube (a room's voxels fit 10 bits an axis)
+        n = len(pos)
+        order = torch.sort((cube[:, 2] << 20) + (cube[:, 1] << 10) + cube[:, 0], stable=True)[1][:, None]
+        for name, v, k in (("pos", pos, 9), ("keys", keys, 12), ("cube", cube, 3)):
+            torch.gather(v.view(n, k), 0, order.expand(n, k), out=out[name][:n].view(n, k))
         return out
     if kind in ("live", "lidar"):
         for _, sensor, T, depth, _ in frames:

@@ -119,8 +119,8 @@ enum { TSDF_SENSOR_PINHOLE = 0, TSDF_SENSOR_LIDAR = 1 };
  * LiDAR images at the nearest beam instead of guarded bilinear;
  * lidar_guard is the bilinear foreground/background threshold in metres
  * (<= 0: the truncation distance).  Launch-shape knobs (results do not
- * depend on them): alloc_tile_h is the pixel-tile height of the allocation
- * kernel, 16 or 32 (0 = chosen from the pixels per launch);
+ * depend on them): alloc_tile_h selects the allocation kernel's pixel tiles,
+ * 16 (small ones) or 32 (large ones; 0 = chosen from the pixels per launch);
  * integrate_ctas_per_sm is the integration kernel's resident CTAs per SM
  * (0 = as many as fit).  For integrate_batch the first map's knobs apply.
  * layer selects the update functor (all maps of one integrate_batch call

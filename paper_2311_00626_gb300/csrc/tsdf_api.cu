@@ -337,8 +337,22 @@ size_t voxel_size_bytes(int storage) {
   return storage == gbt::kStorageColor ? 16 : storage == TSDF_STORAGE_FP32 ? 8 : 4;  // FP16, fixed 16, occupancy
 }
 
-int alloc_ctas(const FrameDev& F, int tile_h) {
-  return ((F.width + gbt::kTileW - 1) / gbt::kTileW) * ((F.height + tile_h - 1) / tile_h);
+int alloc_ctas(const FrameDev& F, gbt::AllocShape shape) {
+  const bool patch = shape.patch && F.kind == TSDF_SENSOR_PINHOLE;
+  const int w = patch ? shape.patch : gbt::kTileW, h = patch ? shape.patch : shape.row_h;
+  return ((F.width + w - 1) / w) * ((F.height + h - 1) / h);
+}
+
+// Numbers the allocation tiles of a batch frame by frame; their count.
+template <class P>
+int number_tiles(P& p, gbt::AllocShape shape) {
+  int ctas = 0;
+  for (int f = 0; f < p.n_frames; ++f) {
+    p.fr[f].vec4 = p.fr[f].width % 4 == 0 && (reinterpret_cast<uintptr_t>(p.fr[f].depth) & 15u) == 0;
+    p.fr[f].blk_begin = ctas;
+    ctas += alloc_ctas(p.fr[f], shape);
+  }
+  return ctas;
 }
 
 int pick_tile_h(int64_t pixels) {
@@ -379,17 +393,17 @@ tsdf_status integrate_one(tsdf_map* m, int kind, const tsdf_pinhole* ph, const t
   p.maps[0] = m->dev;
   tsdf_status st = fill_frame(m, 0, kind, ph, li, depth, rgba, T, p.fr[0]);
   if (st != TSDF_OK) return st;
-  p.fr[0].blk_begin = 0;
   p.fr[0].bit = 0;
   p.fast_rcp = p.fr[0].fast_rcp;
   cudaStream_t s = (cudaStream_t)stream;
   cudaEvent_t* ev = timing_slot(m);
   if (ev) cudaEventRecord(ev[0], s);
-  const int th = m->tile_h ? m->tile_h : pick_tile_h((int64_t)p.fr[0].width * p.fr[0].height);
+  const gbt::AllocShape shape = gbt::pick_alloc_shape(p, m->tile_h);
+  const int ctas = number_tiles(p, shape);
   // one frame per call: each launch may be scheduled while the stream's
   // previous kernel finishes (both kernels wait for it before touching memory)
   p.overlap = 1;
-  if (gbt::launch_band_alloc(p, alloc_ctas(p.fr[0], th), th, s) != cudaSuccess) return cuda_fail();
+  if (gbt::launch_band_alloc(p, ctas, shape, s) != cudaSuccess) return cuda_fail();
   if (ev) {
     cudaEventRecord(ev[1], s);
     cudaEventRecord(ev[2], s);
@@ -671,12 +685,7 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
         pixels += (int64_t)p1.fr[f].width * p1.fr[f].height;
       }
       const int th = lead->tile_h ? lead->tile_h : pick_tile_h(pixels);
-      int ctas = 0;
-      for (int f = 0; f < nf; ++f) {
-        p1.fr[f].blk_begin = ctas;
-        ctas += alloc_ctas(p1.fr[f], th);
-      }
-      p1.alloc_ctas = ctas;
+      p1.alloc_ctas = number_tiles(p1, gbt::AllocShape{0, th});
       p1.wait_extra = lead->wait_extra;
       p1.fast_rcp = 1;
       for (int f = 0; f < nf; ++f) p1.fast_rcp &= p1.fr[f].fast_rcp;
@@ -686,7 +695,9 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
       if (err == cudaErrorNotSupported) {  // not a fused batch: the two kernels
         cudaGetLastError();
         p1.overlap = 1;
-        if (gbt::launch_band_alloc(p1, ctas, th, s) != cudaSuccess) return cuda_fail();
+        const gbt::AllocShape shape = gbt::pick_alloc_shape(p1, lead->tile_h);
+        const int ctas = number_tiles(p1, shape);
+        if (gbt::launch_band_alloc(p1, ctas, shape, s) != cudaSuccess) return cuda_fail();
         if (ev) {
           cudaEventRecord(ev[1], s);
           cudaEventRecord(ev[2], s);
@@ -724,20 +735,14 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
     p.n_frames = nf;
     p.n_maps = n_maps;
     for (int i = 0; i < n_maps; ++i) p.maps[i] = view_set(maps[i], piped ? (b & 1) : 0);
-    int64_t pixels = 0;
     p.fast_rcp = 1;
     for (int f = 0; f < nf; ++f) {
       p.fr[f] = fr[f0 + f];
       p.fr[f].bit = f;
       p.fast_rcp &= p.fr[f].fast_rcp;
-      pixels += (int64_t)p.fr[f].width * p.fr[f].height;
     }
-    const int th = lead->tile_h ? lead->tile_h : pick_tile_h(pixels);
-    int ctas = 0;
-    for (int f = 0; f < nf; ++f) {
-      p.fr[f].blk_begin = ctas;
-      ctas += alloc_ctas(p.fr[f], th);
-    }
+    const gbt::AllocShape shape = gbt::pick_alloc_shape(p, lead->tile_h);
+    const int ctas = number_tiles(p, shape);
     cudaEvent_t* ev = timing_slot(lead);
     if (ev) cudaEventRecord(ev[0], sa);
     if (n_maps == 1) {
@@ -750,7 +755,7 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
     // a single sub-batch runs both kernels back to back on one stream: each
     // may be scheduled while its predecessor drains (see integrate_one)
     p.overlap = p1.overlap = piped ? 0 : 1;
-    if ((n_maps == 1 ? gbt::launch_band_alloc(p1, ctas, th, sa) : gbt::launch_band_alloc(p, ctas, th, sa)) !=
+    if ((n_maps == 1 ? gbt::launch_band_alloc(p1, ctas, shape, sa) : gbt::launch_band_alloc(p, ctas, shape, sa)) !=
         cudaSuccess)
       return cuda_fail();
     if (ev) cudaEventRecord(ev[1], sa);
@@ -1507,10 +1512,9 @@ tsdf_status integrate_depth_static(const tsdf_map_buffers* buf, float voxel_size
   F.fv = intr->fv;
   F.cu = intr->cu;
   F.cv = intr->cv;
-  F.blk_begin = 0;
   F.bit = 0;
   if (!prepare_pose(8.0 * (double)voxel_size, T_world_cam, F)) return TSDF_ERR_ARG;
-  p.fast_rcp = fast_rcp_ok(F, (double)voxel_size, INT_MAX) ? 1 : 0;
+  F.fast_rcp = p.fast_rcp = fast_rcp_ok(F, (double)voxel_size, INT_MAX) ? 1 : 0;
   F.short_walks = short_walks_ok(F, truncation_voxels) ? 1 : 0;
 
   int dev = 0, sms = 0;
@@ -1521,8 +1525,9 @@ tsdf_status integrate_depth_static(const tsdf_map_buffers* buf, float voxel_size
   // the control words must start at zero; a previous call leaves them so,
   // but a call that never ran to completion might not have
   if (cudaMemsetAsync(d.ctl, 0, 4 * sizeof(uint32_t), s) != cudaSuccess) return cuda_fail();
-  const int th = pick_tile_h((int64_t)F.width * F.height);
-  if (gbt::launch_band_alloc(p, alloc_ctas(F, th), th, s) != cudaSuccess) return cuda_fail();
+  const gbt::AllocShape shape = gbt::pick_alloc_shape(p, 0);
+  const int ctas = number_tiles(p, shape);
+  if (gbt::launch_band_alloc(p, ctas, shape, s) != cudaSuccess) return cuda_fail();
   if (gbt::launch_integrate(p, std::max(1, sms) * gbt::integrate_ctas_per_sm(TSDF_STORAGE_FP32), s) !=
       cudaSuccess)
     return cuda_fail();

@@ -20,6 +20,8 @@ constexpr int kTileW = 32;             // allocation CTA = one 32 x (16 or 32) p
 constexpr int kTileHSmall = 16;        // small launches: more CTAs
 constexpr int kTileHBig = 32;          // large launches: fewer, fuller CTAs
 constexpr int kBigTilePixels = 1 << 21;  // pixels per launch from which big tiles are used
+constexpr int kPatchTile = 64;           // patch tiles: 64 x 64 pixels (pick_alloc_shape)
+constexpr int kPatchPixels = 3 << 19;    // pixels per launch from which patch tiles are used
 constexpr int kSetBits = 10;           // CTA-local block-key set: 1024 slots
 constexpr int kSetSize = 1 << kSetBits;
 constexpr int kSetProbes = 32;
@@ -150,6 +152,13 @@ struct FrameDev {
   int32_t bit;           // bit of this frame in the slot masks = its index in the batch
   int32_t fast_rcp;      // host check: this frame's inverted decision values are in [2^-126, 2^126]
   int32_t short_walks;   // host check: this frame's band segments meet fewer than kMaxCells blocks
+  int32_t vec4;          // depth rows can be read as 16-byte words (aligned base, width a multiple of 4)
+};
+
+// Tiles of an allocation launch: pinhole frames in patch x patch pixel tiles
+// (0: in rows like LiDAR frames), the others in kTileW x row_h tiles.
+struct AllocShape {
+  int patch, row_h;
 };
 
 template <int NF, int NM>
@@ -199,8 +208,11 @@ __device__ __forceinline__ int hash_find(const MapDev& m, unsigned long long key
   return -1;
 }
 
+// Tiles for a batch; tile_h: the map's knob (0 = chosen from the batch's pixels).
 template <int NF, int NM>
-cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, int tile_h, cudaStream_t s);
+AllocShape pick_alloc_shape(const BatchParams<NF, NM>& p, int tile_h);
+template <int NF, int NM>
+cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, AllocShape shape, cudaStream_t s);
 template <int NF, int NM>
 cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int n_ctas, cudaStream_t s);
 // Allocation and integration of one batch in a single cooperative launch;

@@ -524,26 +524,27 @@ __global__ void __launch_bounds__(kEsdfThreads)
 // Signed distance (m) at each point: the parent offset's length times the
 // voxel size, negative inside; max_dist for an observed voxel without a
 // parent; NaN for an unknown voxel or a point outside every block.
-__global__ void esdf_query_kernel(const MapDev m, const EsdfDev e, const float* __restrict__ pts,
-                                  int64_t n, float* __restrict__ dist) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float out = __int_as_float(0x7fc00000);
-  const float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
-  const float gx = floorf(__fdiv_rn(x, m.v)), gy = floorf(__fdiv_rn(y, m.v)), gz = floorf(__fdiv_rn(z, m.v));
-  const float lim = 8.0f * 1048576.0f;
-  if (fabsf(gx) < lim && fabsf(gy) < lim && fabsf(gz) < lim) {
-    const int ix = (int)gx, iy = (int)gy, iz = (int)gz;
-    const int p = pool_of(m, ix >> 3, iy >> 3, iz >> 3);
-    if (p >= 0) {
-      const uint32_t s = e.st[(size_t)p * 512 + (ix & 7) + 8 * (iy & 7) + 64 * (iz & 7)];
-      if (s & kEsdfObs) {
-        const float d = (s & kEsdfPar) ? sqrtf((float)dist2(s)) : (float)e.max_dist;
-        out = ((s & kEsdfInside) ? -d : d) * m.v;
-      }
+__global__ void __launch_bounds__(kPointThreads)
+    esdf_query_kernel(const MapDev m, const EsdfDev e, const float* __restrict__ pts, int64_t n, float inv_v,
+                      bool vec, float* __restrict__ dist) {
+  const int64_t i = (int64_t)blockIdx.x * kPointThreads + threadIdx.x;
+  if (kPointsPerThread * i >= n) return;
+  float c[3 * kPointsPerThread], out[kPointsPerThread];
+  int pool[kPointsPerThread], l[kPointsPerThread];
+  load_points(pts, i, n, vec, c);
+  find_points(m, inv_v, c, pool, l);
+  uint32_t st[kPointsPerThread];
+#pragma unroll
+  for (int k = 0; k < kPointsPerThread; ++k) st[k] = pool[k] >= 0 ? e.st[(size_t)pool[k] * 512 + l[k]] : 0u;
+#pragma unroll
+  for (int k = 0; k < kPointsPerThread; ++k) {
+    out[k] = __int_as_float(0x7fc00000);
+    if (st[k] & kEsdfObs) {
+      const float d = (st[k] & kEsdfPar) ? sqrtf((float)dist2(st[k])) : (float)e.max_dist;
+      out[k] = ((st[k] & kEsdfInside) ? -d : d) * m.v;
     }
   }
-  dist[i] = out;
+  store_points(dist, i, n, vec, out);
 }
 
 // ---------------------------------------------------------------- import
@@ -654,8 +655,8 @@ cudaError_t launch_esdf_iteration(const MapDev& m, const EsdfDev& e, int cur, ui
 cudaError_t launch_esdf_query(const MapDev& m, const EsdfDev& e, const float* pts, int64_t n,
                               float* dist, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int threads = 256;
-  esdf_query_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(m, e, pts, n, dist);
+  const PointLaunch q = point_launch(m.v, n, pts, dist, nullptr);
+  esdf_query_kernel<<<q.blocks, kPointThreads, 0, s>>>(m, e, pts, n, q.inv_v, q.vec, dist);
   return cudaGetLastError();
 }
 

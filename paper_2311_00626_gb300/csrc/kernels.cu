@@ -1506,68 +1506,74 @@ __global__ void __launch_bounds__(kFusedThreads, 4)
 }
 
 template <int STORAGE>
-__global__ void query_kernel(const MapDev m, const float* __restrict__ pts, int64_t n,
-                             float* __restrict__ dist, float* __restrict__ weight) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float outD = 0.0f, outW = 0.0f;
-  const float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
-  const float gx = floorf(__fdiv_rn(x, m.v)), gy = floorf(__fdiv_rn(y, m.v)), gz = floorf(__fdiv_rn(z, m.v));
-  const float lim = 8.0f * 1048576.0f;
-  if (fabsf(gx) < lim && fabsf(gy) < lim && fabsf(gz) < lim) {
-    const int ix = (int)gx, iy = (int)gy, iz = (int)gz;
-    const int slot = hash_find(m, pack_key(ix >> 3, iy >> 3, iz >> 3));
-    if (slot >= 0) {
-      const int val = m.vals[slot];
-      if (val >= 0) {
-        const int l = (ix & 7) + 8 * (iy & 7) + 64 * (iz & 7);
-        if (STORAGE == kStorageOcc) {
-          outD = reinterpret_cast<const float*>(m.pool)[(size_t)val * 512 + l];
-        } else if (STORAGE == kStorageF32) {
-          const float2 v = reinterpret_cast<const float2*>(m.pool)[(size_t)val * 512 + l];
-          outD = v.x;
-          outW = v.y;
-        } else if (STORAGE == kStorageX16) {
-          const uint32_t w = reinterpret_cast<const uint32_t*>(m.pool)[(size_t)val * 512 + l];
-          outD = x16_dist(w, m.x16_unit);
-          outW = x16_weight(w);
-        } else {
-          const __half2 h = reinterpret_cast<const __half2*>(m.pool)[(size_t)val * 512 + l];
-          outD = __low2float(h) * m.tau;
-          outW = __high2float(h);
-        }
-      }
+__global__ void __launch_bounds__(kPointThreads)
+    query_kernel(const MapDev m, const float* __restrict__ pts, int64_t n, float inv_v, bool vec,
+                 float* __restrict__ dist, float* __restrict__ weight) {
+  const int64_t i = (int64_t)blockIdx.x * kPointThreads + threadIdx.x;
+  if (kPointsPerThread * i >= n) return;
+  float c[3 * kPointsPerThread], D[kPointsPerThread], W[kPointsPerThread];
+  int pool[kPointsPerThread], l[kPointsPerThread];
+  load_points(pts, i, n, vec, c);
+  find_points(m, inv_v, c, pool, l);
+#pragma unroll
+  for (int k = 0; k < kPointsPerThread; ++k) {
+    D[k] = W[k] = 0.0f;
+    if (pool[k] < 0) continue;
+    const size_t at = (size_t)pool[k] * 512 + l[k];
+    if (STORAGE == kStorageOcc) {
+      D[k] = reinterpret_cast<const float*>(m.pool)[at];
+    } else if (STORAGE == kStorageF32) {
+      const float2 v = reinterpret_cast<const float2*>(m.pool)[at];
+      D[k] = v.x;
+      W[k] = v.y;
+    } else if (STORAGE == kStorageX16) {
+      const uint32_t w = reinterpret_cast<const uint32_t*>(m.pool)[at];
+      D[k] = x16_dist(w, m.x16_unit);
+      W[k] = x16_weight(w);
+    } else {
+      const __half2 h = reinterpret_cast<const __half2*>(m.pool)[at];
+      D[k] = __low2float(h) * m.tau;
+      W[k] = __high2float(h);
     }
   }
-  dist[i] = outD;
-  weight[i] = outW;
+  store_points(dist, i, n, vec, D);
+  store_points(weight, i, n, vec, W);
 }
 
 // Colour of the voxel holding each point: r, g, b and the colour weight;
 // zeros where no block or no colour update exists.
-__global__ void query_color_kernel(const MapDev m, const float* __restrict__ pts, int64_t n,
-                                   float* __restrict__ rgb, float* __restrict__ weight) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float4 out = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  const float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
-  const float gx = floorf(__fdiv_rn(x, m.v)), gy = floorf(__fdiv_rn(y, m.v)), gz = floorf(__fdiv_rn(z, m.v));
-  const float lim = 8.0f * 1048576.0f;
-  if (fabsf(gx) < lim && fabsf(gy) < lim && fabsf(gz) < lim) {
-    const int ix = (int)gx, iy = (int)gy, iz = (int)gz;
-    const int slot = hash_find(m, pack_key(ix >> 3, iy >> 3, iz >> 3));
-    if (slot >= 0) {
-      const int val = m.vals[slot];
-      if (val >= 0) {
-        const int l = (ix & 7) + 8 * (iy & 7) + 64 * (iz & 7);
-        out = reinterpret_cast<const float4*>(m.pool)[(size_t)val * 512 + l];
-      }
-    }
+__global__ void __launch_bounds__(kPointThreads)
+    query_color_kernel(const MapDev m, const float* __restrict__ pts, int64_t n, float inv_v, bool vec,
+                       float* __restrict__ rgb, float* __restrict__ weight) {
+  const int64_t i = (int64_t)blockIdx.x * kPointThreads + threadIdx.x;
+  if (kPointsPerThread * i >= n) return;
+  float c[3 * kPointsPerThread], W[kPointsPerThread];
+  float4 out[kPointsPerThread];
+  int pool[kPointsPerThread], l[kPointsPerThread];
+  load_points(pts, i, n, vec, c);
+  find_points(m, inv_v, c, pool, l);
+#pragma unroll
+  for (int k = 0; k < kPointsPerThread; ++k) {
+    out[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (pool[k] >= 0) out[k] = reinterpret_cast<const float4*>(m.pool)[(size_t)pool[k] * 512 + l[k]];
+    W[k] = out[k].w;
   }
-  rgb[3 * i] = out.x;
-  rgb[3 * i + 1] = out.y;
-  rgb[3 * i + 2] = out.z;
-  weight[i] = out.w;
+  if (vec && kPointsPerThread * (i + 1) <= n) {
+    float4* o = reinterpret_cast<float4*>(rgb) + 3 * i;
+    __stcs(o, make_float4(out[0].x, out[0].y, out[0].z, out[1].x));
+    __stcs(o + 1, make_float4(out[1].y, out[1].z, out[2].x, out[2].y));
+    __stcs(o + 2, make_float4(out[2].z, out[3].x, out[3].y, out[3].z));
+  } else {
+#pragma unroll
+    for (int k = 0; k < kPointsPerThread; ++k)
+      if (kPointsPerThread * i + k < n) {
+        float* o = rgb + 3 * (kPointsPerThread * i + k);
+        o[0] = out[k].x;
+        o[1] = out[k].y;
+        o[2] = out[k].z;
+      }
+  }
+  store_points(weight, i, n, vec, W);
 }
 
 // Occupancy decay over every allocated block: log-odds above 0 drop by
@@ -1798,25 +1804,23 @@ template cudaError_t launch_integrate<kMaxFrames, kMaxMaps>(const BatchParams<kM
 cudaError_t launch_query(const MapDev& m, const float* pts, int64_t n, float* dist, float* weight,
                          cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int threads = 256;
-  const unsigned blocks = (unsigned)((n + threads - 1) / threads);
+  const PointLaunch q = point_launch(m.v, n, pts, dist, weight);
   if (m.storage == kStorageOcc)
-    query_kernel<kStorageOcc><<<blocks, threads, 0, s>>>(m, pts, n, dist, weight);
+    query_kernel<kStorageOcc><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
   else if (m.storage == kStorageF16)
-    query_kernel<kStorageF16><<<blocks, threads, 0, s>>>(m, pts, n, dist, weight);
+    query_kernel<kStorageF16><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
   else if (m.storage == kStorageX16)
-    query_kernel<kStorageX16><<<blocks, threads, 0, s>>>(m, pts, n, dist, weight);
+    query_kernel<kStorageX16><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
   else
-    query_kernel<kStorageF32><<<blocks, threads, 0, s>>>(m, pts, n, dist, weight);
+    query_kernel<kStorageF32><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
   return cudaGetLastError();
 }
 
 cudaError_t launch_query_color(const MapDev& m, const float* pts, int64_t n, float* rgb, float* weight,
                                cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int threads = 256;
-  const unsigned blocks = (unsigned)((n + threads - 1) / threads);
-  query_color_kernel<<<blocks, threads, 0, s>>>(m, pts, n, rgb, weight);
+  const PointLaunch q = point_launch(m.v, n, pts, rgb, weight);
+  query_color_kernel<<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, rgb, weight);
   return cudaGetLastError();
 }
 

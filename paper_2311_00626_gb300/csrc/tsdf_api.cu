@@ -573,10 +573,7 @@ tsdf_status map_create_ex(float voxel_size, int32_t truncation_voxels, float max
     ok = cudaEventCreateWithFlags(&m->ev_alloc[i], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&m->ev_int[i], cudaEventDisableTiming) == cudaSuccess;
   if (ok)
-    ok = gbt::launch_reset(d, m->cap, 0) == cudaSuccess &&
-         cudaMemsetAsync(m->mask1, 0, sizeof(uint32_t) * cap, 0) == cudaSuccess &&
-         cudaMemsetAsync(m->ctl1, 0, sizeof(unsigned int) * 4, 0) == cudaSuccess &&
-         cudaMemsetAsync(d.dirty, 0, (size_t)o.max_blocks, 0) == cudaSuccess &&
+    ok = gbt::launch_reset(d, m->cap, m->mask1, m->ctl1, 0) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;
   if (!ok) {
     free_map(m);
@@ -1381,15 +1378,8 @@ tsdf_status map_reset(tsdf_map* map, void* cuda_stream) {
   if (!map) return TSDF_ERR_ARG;
   if (!on_device(map)) return TSDF_ERR_STATE;
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  if (gbt::launch_reset(map->dev, map->cap, s) != cudaSuccess ||
-      cudaMemsetAsync(map->mask1, 0, sizeof(uint32_t) * map->cap, s) != cudaSuccess ||
-      cudaMemsetAsync(map->ctl1, 0, sizeof(unsigned int) * 4, s) != cudaSuccess ||
-      cudaMemsetAsync(map->dev.dirty, 0, (size_t)map->max_blocks, s) != cudaSuccess)
-    return cuda_fail();
-  if (map->esdf_on &&
-      (cudaMemsetAsync(map->esdf.st, 0, sizeof(uint32_t) * 512 * map->max_blocks, s) != cudaSuccess ||
-       cudaMemsetAsync(map->esdf.stats, 0, sizeof(unsigned long long) * 4, s) != cudaSuccess))
-    return cuda_fail();
+  if (map->esdf_on && gbt::launch_esdf_reset(map->dev, map->esdf, s) != cudaSuccess) return cuda_fail();
+  if (gbt::launch_reset(map->dev, map->cap, map->mask1, map->ctl1, s) != cudaSuccess) return cuda_fail();
   map->status_seen = 0;
   map->frames = 0;
   return TSDF_OK;

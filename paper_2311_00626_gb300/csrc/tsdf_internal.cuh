@@ -338,8 +338,11 @@ cudaError_t launch_query_color(const MapDev& m, const float* pts, int64_t n, flo
                                cudaStream_t s);
 cudaError_t launch_query(const MapDev& m, const float* pts, int64_t n, float* dist, float* weight,
                          cudaStream_t s);
-cudaError_t launch_reset(const MapDev& m, uint32_t cap, cudaStream_t s);
+cudaError_t launch_reset(const MapDev& m, uint32_t cap, uint32_t* mask1, unsigned int* ctl1, cudaStream_t s);
 cudaError_t launch_decay(const MapDev& m, float d_occ, float d_free, cudaStream_t s);
+// Forget the ESDF states of the map's blocks; before launch_reset, which
+// forgets how many there are.
+cudaError_t launch_esdf_reset(const MapDev& m, const EsdfDev& e, cudaStream_t s);
 // ESDF stages (esdf.cu); `cur` selects the current update set.
 cudaError_t launch_esdf_mark(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);
 cudaError_t launch_esdf_clear(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);

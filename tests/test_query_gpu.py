@@ -107,3 +107,30 @@ def test_color_and_esdf_queries_match_exports(n):
         m.esdf_query(pts, out)
         np.testing.assert_array_equal(out.cpu().numpy(), want[0])
     m.close()
+
+
+@pytest.mark.parametrize("max_blocks", [1, 7, 33, 1 << 12])
+def test_reset_leaves_nothing_behind(max_blocks):
+    """After a reset a map (its table, pool, changed flags, ESDF states) behaves like a new one."""
+    import paper_2311_00626_gb300 as gt
+    rng = np.random.default_rng(max_blocks)
+    n = min(max_blocks, 60)
+    keys = np.stack([np.arange(n), np.zeros(n), np.zeros(n)], 1).astype(np.int32)
+    D = rng.uniform(-0.2, 0.2, (2, n, 512)).astype(np.float32)
+    W = np.ones((n, 512), np.float32)
+    a = gt.TsdfMap(0.05, 4, 100.0, max_blocks=max_blocks)
+    a.import_blocks(keys, D[0], W)
+    a.esdf_update()
+    a.reset()
+    assert a.num_blocks() == 0 and a.esdf_stats() == dict(iterations=0, swept=0, pulled=0, cleared=0)
+    b = gt.TsdfMap(0.05, 4, 100.0, max_blocks=max_blocks)
+    half = max(1, n // 2)
+    for m in (a, b):
+        m.import_blocks(keys[:half], D[1, :half], W[:half])
+        m.esdf_update()
+        assert m.sync() == 0
+    for x, y in zip(a.export() + a.esdf_export(), b.export() + b.esdf_export()):
+        np.testing.assert_array_equal(x, y)
+    assert a.esdf_stats() == b.esdf_stats()
+    a.close()
+    b.close()

@@ -26,6 +26,7 @@
 // Discrete decisions use explicit round-to-nearest intrinsics in a fixed
 // order (no contraction) so that they are reproducible on a CPU.
 #include <algorithm>
+#include <atomic>
 #include <cfloat>
 
 #include "tsdf_internal.cuh"
@@ -44,6 +45,13 @@ __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol
 
 constexpr float kPiF = (float)3.14159265358979323846;
 constexpr float kHalfPiF = (float)(3.14159265358979323846 / 2);
+
+// Approximate reciprocal (within 1 ulp; 0 gives +-inf).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 // IEEE round-to-nearest reciprocal of a decision input.  FAST: the hardware
 // approximation (within 1 ulp) refined by one Newton step with fused
@@ -477,13 +485,6 @@ __device__ __forceinline__ bool bitmap_insert(uint32_t* bm, uint32_t* keys, uint
     keys[i] = key;
   }
   return true;
-}
-
-// Approximate reciprocal (within 1 ulp; 0 gives +-inf).
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
 }
 
 // Whether every block that the bundle can meet is in the bitmap.  ow: sensor
@@ -922,257 +923,279 @@ __device__ __forceinline__ void apply_color(const MapDev& m, float& R, float& G,
   W = fminf(wn, m.wmax);
 }
 
-// A thread's four voxels in registers: D and W (TSDF distance and weight,
-// occupancy log-odds, or colour red and weight) and, for colour only, G and B.
+// A thread's four voxels: (x, y, z), (x, y, z + 1), (x + 1, y, z) and
+// (x + 1, y, z + 1), as global voxel indices in FP32 (exact: below 2^23 + 8
+// in magnitude), and the index `at` of the first two's x pair in its block
+// (x / 2 + 4 y + 32 z).  A warp holds two z layers, 8 x 8 voxels each, and its
+// lanes look one layer up at a time: a gather of depths then touches fewer
+// image rows than with four voxels along x per thread (two layers at a time).
+struct VoxelQuad {
+  float x, y, z;
+  int at;
+};
+
+// The voxels in registers: D and W (TSDF distance and weight, occupancy
+// log-odds, or colour red and weight) and, for colour only, G and B.
 template <int STORAGE>
 struct Voxels4;
 
 template <>
 struct Voxels4<kStorageF32> {
-  __device__ __forceinline__ static void load(const MapDev& m, int pool, int t, float* D, float* W,
+  __device__ __forceinline__ static void load(const MapDev& m, int pool, int at, float* D, float* W,
                                               float* G, float* B) {
-    const float4* src = reinterpret_cast<const float4*>(m.pool) + (size_t)pool * 256 + 2 * t;
-    const float4 a = src[0], b = src[1];
-    D[0] = a.x; W[0] = a.y; D[1] = a.z; W[1] = a.w;
-    D[2] = b.x; W[2] = b.y; D[3] = b.z; W[3] = b.w;
+    const float4* src = reinterpret_cast<const float4*>(m.pool) + (size_t)pool * 256 + at;
+    const float4 a = src[0], b = src[32];
+    D[0] = a.x; W[0] = a.y; D[2] = a.z; W[2] = a.w;
+    D[1] = b.x; W[1] = b.y; D[3] = b.z; W[3] = b.w;
   }
-  __device__ __forceinline__ static void store(const MapDev& m, int pool, int t, const float* D,
+  __device__ __forceinline__ static void store(const MapDev& m, int pool, int at, const float* D,
                                                const float* W, const float* G, const float* B) {
-    float4* dst = reinterpret_cast<float4*>(m.pool) + (size_t)pool * 256 + 2 * t;
-    dst[0] = make_float4(D[0], W[0], D[1], W[1]);
-    dst[1] = make_float4(D[2], W[2], D[3], W[3]);
+    float4* dst = reinterpret_cast<float4*>(m.pool) + (size_t)pool * 256 + at;
+    dst[0] = make_float4(D[0], W[0], D[2], W[2]);
+    dst[32] = make_float4(D[1], W[1], D[3], W[3]);
   }
 };
 
 template <>
 struct Voxels4<kStorageOcc> {
-  __device__ __forceinline__ static void load(const MapDev& m, int pool, int t, float* D, float* W,
+  __device__ __forceinline__ static void load(const MapDev& m, int pool, int at, float* D, float* W,
                                               float* G, float* B) {
-    const float4 a = reinterpret_cast<const float4*>(m.pool)[(size_t)pool * 128 + t];
-    D[0] = a.x; D[1] = a.y; D[2] = a.z; D[3] = a.w;
+    const float2* src = reinterpret_cast<const float2*>(m.pool) + (size_t)pool * 256 + at;
+    const float2 a = src[0], b = src[32];
+    D[0] = a.x; D[2] = a.y; D[1] = b.x; D[3] = b.y;
     W[0] = W[1] = W[2] = W[3] = 0.0f;
   }
-  __device__ __forceinline__ static void store(const MapDev& m, int pool, int t, const float* D,
+  __device__ __forceinline__ static void store(const MapDev& m, int pool, int at, const float* D,
                                                const float* W, const float* G, const float* B) {
-    reinterpret_cast<float4*>(m.pool)[(size_t)pool * 128 + t] = make_float4(D[0], D[1], D[2], D[3]);
+    float2* dst = reinterpret_cast<float2*>(m.pool) + (size_t)pool * 256 + at;
+    dst[0] = make_float2(D[0], D[2]);
+    dst[32] = make_float2(D[1], D[3]);
   }
 };
 
-template <>
-struct Voxels4<kStorageF16> {
-  __device__ __forceinline__ static void load(const MapDev& m, int pool, int t, float* D, float* W,
-                                              float* G, float* B) {
-    const uint4 raw = reinterpret_cast<const uint4*>(m.pool)[(size_t)pool * 128 + t];
-    const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const __half2 h = *reinterpret_cast<const __half2*>(&w4[i]);
-      D[i] = __low2float(h) * m.tau;
-      W[i] = __high2float(h);
-    }
+// 16-bit storages: one word per voxel.
+template <int STORAGE>
+__device__ __forceinline__ void unpack16(const MapDev& m, uint32_t w, float& D, float& W) {
+  if (STORAGE == kStorageF16) {
+    const __half2 h = *reinterpret_cast<const __half2*>(&w);
+    D = __low2float(h) * m.tau;
+    W = __high2float(h);
+  } else {
+    D = x16_dist(w, m.x16_unit);
+    W = x16_weight(w);
   }
-  __device__ __forceinline__ static void store(const MapDev& m, int pool, int t, const float* D,
+}
+template <int STORAGE>
+__device__ __forceinline__ uint32_t pack16(const MapDev& m, float D, float W) {
+  if (STORAGE == kStorageF16) {
+    const __half2 h = __floats2half2_rn(D * m.inv_tau, W);
+    return *reinterpret_cast<const uint32_t*>(&h);
+  }
+  return x16_pack(D, W, m.x16_scale);
+}
+template <int STORAGE>
+struct Voxels4Word {
+  __device__ __forceinline__ static void load(const MapDev& m, int pool, int at, float* D, float* W,
+                                              float* G, float* B) {
+    const uint2* src = reinterpret_cast<const uint2*>(m.pool) + (size_t)pool * 256 + at;
+    const uint2 a = src[0], b = src[32];
+    unpack16<STORAGE>(m, a.x, D[0], W[0]);
+    unpack16<STORAGE>(m, a.y, D[2], W[2]);
+    unpack16<STORAGE>(m, b.x, D[1], W[1]);
+    unpack16<STORAGE>(m, b.y, D[3], W[3]);
+  }
+  __device__ __forceinline__ static void store(const MapDev& m, int pool, int at, const float* D,
                                                const float* W, const float* G, const float* B) {
-    uint32_t w4[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const __half2 h = __floats2half2_rn(D[i] * m.inv_tau, W[i]);
-      w4[i] = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    reinterpret_cast<uint4*>(m.pool)[(size_t)pool * 128 + t] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    uint2* dst = reinterpret_cast<uint2*>(m.pool) + (size_t)pool * 256 + at;
+    dst[0] = make_uint2(pack16<STORAGE>(m, D[0], W[0]), pack16<STORAGE>(m, D[2], W[2]));
+    dst[32] = make_uint2(pack16<STORAGE>(m, D[1], W[1]), pack16<STORAGE>(m, D[3], W[3]));
   }
 };
-
 template <>
-struct Voxels4<kStorageX16> {
-  __device__ __forceinline__ static void load(const MapDev& m, int pool, int t, float* D, float* W,
-                                              float* G, float* B) {
-    const uint4 raw = reinterpret_cast<const uint4*>(m.pool)[(size_t)pool * 128 + t];
-    const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      D[i] = x16_dist(w4[i], m.x16_unit);
-      W[i] = x16_weight(w4[i]);
-    }
-  }
-  __device__ __forceinline__ static void store(const MapDev& m, int pool, int t, const float* D,
-                                               const float* W, const float* G, const float* B) {
-    reinterpret_cast<uint4*>(m.pool)[(size_t)pool * 128 + t] =
-        make_uint4(x16_pack(D[0], W[0], m.x16_scale), x16_pack(D[1], W[1], m.x16_scale),
-                   x16_pack(D[2], W[2], m.x16_scale), x16_pack(D[3], W[3], m.x16_scale));
-  }
-};
+struct Voxels4<kStorageF16> : Voxels4Word<kStorageF16> {};
+template <>
+struct Voxels4<kStorageX16> : Voxels4Word<kStorageX16> {};
 
 template <>
 struct Voxels4<kStorageColor> {
-  __device__ __forceinline__ static void load(const MapDev& m, int pool, int t, float* D, float* W,
+  __device__ __forceinline__ static void load(const MapDev& m, int pool, int at, float* D, float* W,
                                               float* G, float* B) {
-    const float4* src = reinterpret_cast<const float4*>(m.pool) + (size_t)pool * 512 + 4 * t;
+    const float4* src = reinterpret_cast<const float4*>(m.pool) + (size_t)pool * 512 + 2 * at;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const float4 a = src[i];
+      const float4 a = src[(i & 1) * 64 + (i >> 1)];
       D[i] = a.x; G[i] = a.y; B[i] = a.z; W[i] = a.w;
     }
   }
-  __device__ __forceinline__ static void store(const MapDev& m, int pool, int t, const float* D,
+  __device__ __forceinline__ static void store(const MapDev& m, int pool, int at, const float* D,
                                                const float* W, const float* G, const float* B) {
-    float4* dst = reinterpret_cast<float4*>(m.pool) + (size_t)pool * 512 + 4 * t;
+    float4* dst = reinterpret_cast<float4*>(m.pool) + (size_t)pool * 512 + 2 * at;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) dst[i] = make_float4(D[i], G[i], B[i], W[i]);
+    for (int i = 0; i < 4; ++i) dst[(i & 1) * 64 + (i >> 1)] = make_float4(D[i], G[i], B[i], W[i]);
   }
 };
 
-// A thread's four voxels: block (bx, by, bz), local x = lx0 .. lx0 + 3 at
-// local (ly, lz).
-struct VoxelRow {
-  int bx, by, bz, lx0, ly, lz;
-};
-
-// Voxel centres of a row in frame F's sensor frame (Eq. 1), in the FP32
-// decision sequence p_i = fma(R_i0, qx, fma(R_i1, qy, fma(R_i2, qz, t_i))).
-__device__ __forceinline__ void row_points(const FrameDev& F, float v, const VoxelRow& r,
-                                           float* px, float* py, float* pz) {
-  const int rx = (r.bx - F.a[0]) * 8 + r.lx0;
-  const int ry = (r.by - F.a[1]) * 8 + r.ly;
-  const int rz = (r.bz - F.a[2]) * 8 + r.lz;
-  const float qy = __fmul_rn(__fadd_rn((float)ry, 0.5f), v);
-  const float qz = __fmul_rn(__fadd_rn((float)rz, 0.5f), v);
-  const float cx = __fmaf_rn(F.Rcl[1], qy, __fmaf_rn(F.Rcl[2], qz, F.tloc[0]));
-  const float cy = __fmaf_rn(F.Rcl[4], qy, __fmaf_rn(F.Rcl[5], qz, F.tloc[1]));
-  const float cz = __fmaf_rn(F.Rcl[7], qy, __fmaf_rn(F.Rcl[8], qz, F.tloc[2]));
+// Voxel centres in frame F's sensor frame (Eq. 1), in the FP32 decision
+// sequence p_i = fma(R_i0, qx, fma(R_i1, qy, fma(R_i2, qz, t_i))).
+__device__ __forceinline__ void quad_points(const FrameDev& F, float v, const VoxelQuad& r,
+                                            float* px, float* py, float* pz) {
+  // anchor-relative voxel indices: exact in FP32 (|index| < 2^24)
+  const float rx = __fsub_rn(r.x, (float)(F.a[0] * 8)), ry = __fsub_rn(r.y, (float)(F.a[1] * 8)),
+              rz = __fsub_rn(r.z, (float)(F.a[2] * 8));
+  const float qy = __fmul_rn(__fadd_rn(ry, 0.5f), v);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float qx = __fmul_rn(__fadd_rn((float)(rx + i), 0.5f), v);
-    px[i] = __fmaf_rn(F.Rcl[0], qx, cx);
-    py[i] = __fmaf_rn(F.Rcl[3], qx, cy);
-    pz[i] = __fmaf_rn(F.Rcl[6], qx, cz);
+  for (int k = 0; k < 2; ++k) {
+    const float qz = __fmul_rn(__fadd_rn(rz, (float)k + 0.5f), v);
+    const float cx = __fmaf_rn(F.Rcl[1], qy, __fmaf_rn(F.Rcl[2], qz, F.tloc[0]));
+    const float cy = __fmaf_rn(F.Rcl[4], qy, __fmaf_rn(F.Rcl[5], qz, F.tloc[1]));
+    const float cz = __fmaf_rn(F.Rcl[7], qy, __fmaf_rn(F.Rcl[8], qz, F.tloc[2]));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float qx = __fmul_rn(__fadd_rn(rx, (float)j + 0.5f), v);
+      px[2 * j + k] = __fmaf_rn(F.Rcl[0], qx, cx);
+      py[2 * j + k] = __fmaf_rn(F.Rcl[3], qx, cy);
+      pz[2 * j + k] = __fmaf_rn(F.Rcl[6], qx, cz);
+    }
   }
 }
 
 // A pinhole frame's projection constants, staged in shared memory once per
-// CTA: six 16-byte loads per frame in the voxel loop instead of one
-// constant-bank load per field (the frame index is not known at compile
-// time, so the fields cannot be instruction operands).
+// CTA: 16-byte loads in the voxel loop instead of one constant-bank load per
+// field (the frame index is not known at compile time, so the fields cannot
+// be instruction operands).  What multiplies voxel pairs is stored twice, as
+// the paired operations read it.
 struct __align__(16) FrameProj {
-  float4 r0, r1, r2;  // rows of R_CL, with t_loc in w
-  float4 cam;         // fu, fv, cu, cv
-  int4 anchor;        // a, width
-  float4 size;        // width, height (as floats), height (integer bits), unused
+  float2 r0x, r1x, r2x, r0y, r1y, r2y, r0z, r1z, r2z;  // R_CL, duplicated
+  float2 t0, t1, t2, nfu, nfv, cu, cv;                 // t_loc; -fu, -fv
+  float ax, ay, az;                                    // 8 a: the anchor block's first voxel
+  int width;
+  const float* depth;
+  int height, unused;
 };
 
+__device__ __forceinline__ float2 twice(float x) { return make_float2(x, x); }
+
 __device__ __forceinline__ void stage_frame(const FrameDev& F, FrameProj& S) {
-  S.r0 = make_float4(F.Rcl[0], F.Rcl[1], F.Rcl[2], F.tloc[0]);
-  S.r1 = make_float4(F.Rcl[3], F.Rcl[4], F.Rcl[5], F.tloc[1]);
-  S.r2 = make_float4(F.Rcl[6], F.Rcl[7], F.Rcl[8], F.tloc[2]);
-  S.cam = make_float4(F.fu, F.fv, F.cu, F.cv);
-  S.anchor = make_int4(F.a[0], F.a[1], F.a[2], F.width);
-  S.size = make_float4((float)F.width, (float)F.height, __int_as_float(F.height), 0.0f);
+  S.r0x = twice(F.Rcl[0]); S.r1x = twice(F.Rcl[3]); S.r2x = twice(F.Rcl[6]);
+  S.r0y = twice(F.Rcl[1]); S.r1y = twice(F.Rcl[4]); S.r2y = twice(F.Rcl[7]);
+  S.r0z = twice(F.Rcl[2]); S.r1z = twice(F.Rcl[5]); S.r2z = twice(F.Rcl[8]);
+  S.t0 = twice(F.tloc[0]); S.t1 = twice(F.tloc[1]); S.t2 = twice(F.tloc[2]);
+  S.nfu = twice(-F.fu); S.nfv = twice(-F.fv);
+  S.cu = twice(F.cu); S.cv = twice(F.cv);
+  S.ax = (float)(F.a[0] * 8); S.ay = (float)(F.a[1] * 8); S.az = (float)(F.a[2] * 8);
+  S.width = F.width;
+  S.height = F.height;
+  S.depth = F.depth;
 }
 
-// row_points with staged constants (same arithmetic).
-__device__ __forceinline__ void row_points_staged(const float4& r0, const float4& r1, const float4& r2,
-                                                  const int4& an, float v, const VoxelRow& r,
-                                                  float* px, float* py, float* pz) {
-  const int rx = (r.bx - an.x) * 8 + r.lx0;
-  const int ry = (r.by - an.y) * 8 + r.ly;
-  const int rz = (r.bz - an.z) * 8 + r.lz;
-  const float qy = __fmul_rn(__fadd_rn((float)ry, 0.5f), v);
-  const float qz = __fmul_rn(__fadd_rn((float)rz, 0.5f), v);
-  const float cx = __fmaf_rn(r0.y, qy, __fmaf_rn(r0.z, qz, r0.w));
-  const float cy = __fmaf_rn(r1.y, qy, __fmaf_rn(r1.z, qz, r1.w));
-  const float cz = __fmaf_rn(r2.y, qy, __fmaf_rn(r2.z, qz, r2.w));
-  const float fx = (float)rx;  // rx + i is exact in FP32 (|rx| < 2^24)
-  // voxel pairs on the paired FP32 operations (per component the same
-  // round-to-nearest result as the scalar ones)
-  const float2 half = make_float2(0.5f, 0.5f), vv = make_float2(v, v);
-  const float2 c0 = make_float2(cx, cx), c1 = make_float2(cy, cy), c2 = make_float2(cz, cz);
-  const float2 a0 = make_float2(r0.x, r0.x), a1 = make_float2(r1.x, r1.x), a2 = make_float2(r2.x, r2.x);
-#pragma unroll
-  for (int i = 0; i < 4; i += 2) {
-    const float2 qx = __fmul2_rn(__fadd2_rn(__fadd2_rn(make_float2(fx, fx), make_float2((float)i, (float)(i + 1))),
-                                            half), vv);
-    const float2 x = __ffma2_rn(a0, qx, c0), y = __ffma2_rn(a1, qx, c1), z = __ffma2_rn(a2, qx, c2);
-    px[i] = x.x; px[i + 1] = x.y;
-    py[i] = y.x; py[i + 1] = y.y;
-    pz[i] = z.x; pz[i + 1] = z.y;
-  }
+// -1 / z of a voxel pair, the negative of rcp_dec<FAST> (rounding is
+// symmetric in sign): e = 1 + z y with y ~ -1/z, then y + y e.
+template <bool FAST>
+__device__ __forceinline__ float2 neg_rcp2(float2 z) {
+  if (!FAST) return make_float2(-__frcp_rn(z.x), -__frcp_rn(z.y));
+  const float2 y = make_float2(rcp_approx(-z.x), rcp_approx(-z.y));
+  return __ffma2_rn(y, __ffma2_rn(z, y, twice(1.0f)), y);
 }
 
-// PAIRED_RCP: the projection reciprocals refined on the paired operations
-// (pinhole-only kernels; in the kernels with the LiDAR path it raised the
-// register count from 72 to 79, one resident CTA per SM fewer).
+// floor(u) by a round-down addition: the low bits of u + 1.5 * 2^23 hold it
+// for |u| < 2^22, and for any other u (NaN included) the difference from
+// kFloorBits is, unsigned, at least 2^22.  (A conversion instruction runs at an
+// eighth of the rate, on the unit that also serves the reciprocals.)
+constexpr float kFloorMagic = 12582912.0f;
+constexpr uint32_t kFloorBits = 0x4B400000u;
+
 // NQ consecutive pinhole frames of the batch: phase 1 projects every voxel
 // into every frame (Eq. 2, nearest pixel) and issues all depth loads (and
 // colour loads for a colour layer), phase 2 applies the updates in frame
 // order.  An out-of-image projection reads no pixel and yields d = 0, which
 // is invalid like a missing depth.  A colour layer updates only voxels within
-// tau of the surface on both sides.
-template <int NQ, int STORAGE, bool WEIGHTED, bool FAST, bool PAIRED_RCP, class P>
-__device__ __forceinline__ void fuse_pinhole(const P& p, const FrameProj* s_fp, const int (&fq)[4],
-                                             const MapDev& m, const VoxelRow& r, float* D, float* W,
-                                             float* G, float* B, unsigned long long& upd) {
+// tau of the surface on both sides.  Voxel pairs share the paired FP32
+// operations (per component the same round-to-nearest result), and the
+// constant-weight update is computed for every voxel and selected, not
+// branched to, so the four voxels' chains overlap.
+template <int NQ, int STORAGE, bool WEIGHTED, bool FAST, class P>
+__device__ __forceinline__ void fuse_pinhole(const P& p, const FrameProj* s_fp, const int (&fq)[2],
+                                             const MapDev& m, const VoxelQuad& r, float* D, float* W,
+                                             float* G, float* B, uint32_t& upd) {
   float d[NQ][4], z[NQ][4];
   uint32_t c[NQ][4];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     const FrameProj& S = s_fp[fq[q]];
-    const float4 r0 = S.r0, r1 = S.r1, r2 = S.r2, cam = S.cam, size = S.size;
-    const int4 an = S.anchor;
-    const float* depth = p.fr[fq[q]].depth;
-    float px[4], py[4];
-    row_points_staged(r0, r1, r2, an, m.v, r, px, py, z[q]);
-    // pixel coordinates of voxel pairs on the paired FP32 operations
-    float uu[4], vv[4];
-    const float2 fu2 = make_float2(cam.x, cam.x), cu2 = make_float2(cam.z, cam.z);
-    const float2 fv2 = make_float2(cam.y, cam.y), cv2 = make_float2(cam.w, cam.w);
-    const float2 half = make_float2(0.5f, 0.5f);
+    const float* depth = S.depth;
+    const int width = S.width, height = S.height;
+    // voxel centres in the sensor frame (quad_points with staged constants),
+    // as pairs along z
+    const float2 qy = twice(__fmul_rn(__fadd_rn(__fsub_rn(r.y, S.ay), 0.5f), m.v));
+    const float2 qz = __fmul2_rn(__fadd2_rn(twice(__fsub_rn(r.z, S.az)), make_float2(0.5f, 1.5f)), twice(m.v));
+    const float2 cx = __ffma2_rn(S.r0y, qy, __ffma2_rn(S.r0z, qz, S.t0));
+    const float2 cy = __ffma2_rn(S.r1y, qy, __ffma2_rn(S.r1z, qz, S.t1));
+    const float2 cz = __ffma2_rn(S.r2y, qy, __ffma2_rn(S.r2z, qz, S.t2));
+    const float fx = __fsub_rn(r.x, S.ax);
 #pragma unroll
     for (int i = 0; i < 4; i += 2) {
-      const float2 iz = PAIRED_RCP ? rcp_dec2<FAST>(z[q][i], z[q][i + 1])
-                                   : make_float2(rcp_dec<FAST>(z[q][i]), rcp_dec<FAST>(z[q][i + 1]));
-      const float2 u = __fadd2_rn(__ffma2_rn(__fmul2_rn(make_float2(px[i], px[i + 1]), iz), fu2, cu2), half);
-      const float2 v = __fadd2_rn(__ffma2_rn(__fmul2_rn(make_float2(py[i], py[i + 1]), iz), fv2, cv2), half);
-      uu[i] = u.x; uu[i + 1] = u.y;
-      vv[i] = v.x; vv[i + 1] = v.y;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float u = uu[i], v = vv[i];
-      bool in;
-      int pix;
+      const float2 qx = twice(__fmul_rn(__fadd_rn(fx, (float)(i / 2) + 0.5f), m.v));
+      const float2 x = __ffma2_rn(S.r0x, qx, cx), y = __ffma2_rn(S.r1x, qx, cy), zz = __ffma2_rn(S.r2x, qx, cz);
+      const float2 niz = neg_rcp2<FAST>(zz);
+      // u = x / z fu + cu + 1/2 as (x (-1/z)) (-fu) + cu + 1/2
+      const float2 u = __fadd2_rn(__ffma2_rn(__fmul2_rn(x, niz), S.nfu, S.cu), twice(0.5f));
+      const float2 v = __fadd2_rn(__ffma2_rn(__fmul2_rn(y, niz), S.nfv, S.cv), twice(0.5f));
+      z[q][i] = zz.x;
+      z[q][i + 1] = zz.y;
       if (FAST) {
         // pixel = floor(u), valid iff 0 <= u < W: one unsigned comparison of
-        // the floored value per axis (u is finite here: z > 0 implies
-        // z >= 2^-126 in FAST batches, so 1 / z is finite)
-        const int iu = __float2int_rd(u), iv = __float2int_rd(v);
-        in = z[q][i] > 0.0f && (unsigned)iu < (unsigned)an.w && (unsigned)iv < (unsigned)__float_as_int(size.z);
-        pix = iv * an.w + iu;
+        // the floored value per axis (the host checked W, H <= 2^22; z > 0
+        // implies z >= 2^-126 in FAST batches, so 1 / z is finite)
+        const float2 tu = __fadd2_rd(u, twice(kFloorMagic)), tv = __fadd2_rd(v, twice(kFloorMagic));
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const uint32_t iu = __float_as_uint(k ? tu.y : tu.x) - kFloorBits;
+          const uint32_t iv = __float_as_uint(k ? tv.y : tv.x) - kFloorBits;
+          const bool in = z[q][i + k] > 0.0f && iu < (uint32_t)width && iv < (uint32_t)height;
+          const int pix = (int)iv * width + (int)iu;
+          d[q][i + k] = in ? __ldg(depth + pix) : 0.0f;
+          if (STORAGE == kStorageColor) c[q][i + k] = in ? __ldg(p.fr[fq[q]].rgba + pix) : 0u;
+        }
       } else {
-        in = z[q][i] > 0.0f && u >= 0.0f && u < size.x && v >= 0.0f && v < size.y;
-        pix = (int)v * an.w + (int)u;
-      }
-      if (STORAGE == kStorageColor) {
-        d[q][i] = in ? __ldg(depth + pix) : 0.0f;
-        c[q][i] = in ? __ldg(p.fr[fq[q]].rgba + pix) : 0u;
-      } else {
-        d[q][i] = in ? __ldg(depth + pix) : 0.0f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float uk = k ? u.y : u.x, vk = k ? v.y : v.x;
+          const bool in = z[q][i + k] > 0.0f && uk >= 0.0f && uk < (float)width && vk >= 0.0f && vk < (float)height;
+          const int pix = (int)vk * width + (int)uk;
+          d[q][i + k] = in ? __ldg(depth + pix) : 0.0f;
+          if (STORAGE == kStorageColor) c[q][i + k] = in ? __ldg(p.fr[fq[q]].rgba + pix) : 0u;
+        }
       }
     }
   }
 #pragma unroll
   for (int q = 0; q < NQ; ++q)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float dp = __fsub_rn(d[q][i], z[q][i]);
+    for (int i = 0; i < 4; i += 2) {
+      const float2 dp = __ffma2_rn(make_float2(z[q][i], z[q][i + 1]), twice(-1.0f),
+                                   make_float2(d[q][i], d[q][i + 1]));  // d - z, rounded once
       // a valid depth, 0 < d <= FLT_MAX: one unsigned comparison of its bits
-      if ((__float_as_uint(d[q][i]) - 1u) < 0x7F7FFFFFu && !(dp < -m.tau)) {
-        if (STORAGE == kStorageColor) {
-          if (dp > m.tau) continue;
+      const bool ok0 = depth_ok(d[q][i]) && !(dp.x < -m.tau), ok1 = depth_ok(d[q][i + 1]) && !(dp.y < -m.tau);
+      if (STORAGE == kStorageColor) {
+        if (ok0 && !(dp.x > m.tau)) {
           apply_color(m, D[i], G[i], B[i], W[i], c[q][i]);
-        } else {
-          apply<STORAGE, WEIGHTED>(m, D[i], W[i], z[q][i], dp);
+          ++upd;
         }
-        ++upd;
+        if (ok1 && !(dp.y > m.tau)) {
+          apply_color(m, D[i + 1], G[i + 1], B[i + 1], W[i + 1], c[q][i + 1]);
+          ++upd;
+        }
+      } else if (STORAGE == kStorageOcc || WEIGHTED) {
+        if (ok0) apply<STORAGE, WEIGHTED>(m, D[i], W[i], z[q][i], dp.x);
+        if (ok1) apply<STORAGE, WEIGHTED>(m, D[i + 1], W[i + 1], z[q][i + 1], dp.y);
+        upd += (ok0 ? 1u : 0u) + (ok1 ? 1u : 0u);
+      } else {
+        const float2 wn = __fadd2_rn(make_float2(W[i], W[i + 1]), twice(1.0f));
+        const float2 D2 = make_float2(D[i], D[i + 1]);
+        const float2 diff = __ffma2_rn(D2, twice(-1.0f), make_float2(fminf(dp.x, m.tau), fminf(dp.y, m.tau)));
+        const float2 dn = __fadd2_rn(D2, __fmul2_rn(diff, make_float2(rcp_approx(wn.x), rcp_approx(wn.y))));
+        if (ok0) { D[i] = dn.x; W[i] = fminf(wn.x, m.wmax); ++upd; }
+        if (ok1) { D[i + 1] = dn.y; W[i + 1] = fminf(wn.y, m.wmax); ++upd; }
       }
     }
 }
@@ -1183,11 +1206,11 @@ __device__ __forceinline__ void fuse_pinhole(const P& p, const FrameProj* s_fp, 
 // sensor origin, outside the elevation rows or with an invalid sample is not
 // updated; azimuth wraps.  Colour layers take pinhole frames only.
 template <int STORAGE, bool WEIGHTED>
-__device__ __forceinline__ void fuse_lidar(const FrameDev& F, const MapDev& m, const VoxelRow& r,
-                                           float* D, float* W, unsigned long long& upd) {
+__device__ __forceinline__ void fuse_lidar(const FrameDev& F, const MapDev& m, const VoxelQuad& r,
+                                           float* D, float* W, uint32_t& upd) {
   if (STORAGE == kStorageColor) return;
   float px[4], py[4], pz[4];
-  row_points(F, m.v, r, px, py, pz);
+  quad_points(F, m.v, r, px, py, pz);
   const int naz = F.width, nel = F.height;
   float rr[4], th[4], ph[4], fx[4], fy[4], d00[4], d10[4], d01[4], d11[4];
   bool ok[4];
@@ -1267,29 +1290,29 @@ __device__ __forceinline__ void fuse_lidar(const FrameDev& F, const MapDev& m, c
   }
 }
 
-// Shared memory of the integration workers of a CTA: G groups of
-// kIntegrateThreads threads, each group working on its own work-list
-// entries.
-template <int NF, int NM, int G>
+// Shared memory of the integration workers of a CTA.
+constexpr int kRing = 8;  // entries in hand
+template <int NF, int NM>
 struct IntegSmem {
   uint32_t begin[NM + 1];         // first entry of each map's list in the batch's work
   unsigned long long upd[NM];     // voxel updates per map
   unsigned long long pairs[NM];   // (block, frame) pairs per map
-  uint32_t next[G][2];            // per group: the entry in hand and the next one
+  uint32_t ticket;                // slabs handed out
+  uint32_t seq[kRing];            // sequence number of the entry in a ring slot
+  uint32_t entry[kRing];
+  uint32_t done[kRing];           // slabs finished in the slot's entries, all together
   FrameProj fp[NF];
 };
 
-// Barrier of the kIntegrateThreads threads of worker group g: the CTA
-// barrier when the CTA is one group, else hardware barrier 1 + g.
-template <int G>
-__device__ __forceinline__ void group_sync(int g) {
-  if (G == 1) {
-    __syncthreads();
-  } else if (g == 0) {
-    asm volatile("bar.sync 1, %0;" ::"n"(kIntegrateThreads) : "memory");
-  } else {
-    asm volatile("bar.sync 2, %0;" ::"n"(kIntegrateThreads) : "memory");
-  }
+// Wait until *a == value (a shared-memory word that another warp of the CTA
+// sets without waiting for this one); false after 2^22 polls.
+__device__ __forceinline__ bool poll_shared(const uint32_t* a, uint32_t value) {
+  for (int i = 0; i < (1 << 22); ++i)
+    if (*(const volatile uint32_t*)a == value) {
+      __threadfence_block();
+      return true;
+    }
+  return false;
 }
 
 // Entry metadata: COHERENT loads bypass L1, for a kernel that reads
@@ -1303,19 +1326,30 @@ __device__ __forceinline__ T meta_load(const T* a) {
 // The integration of a batch's work list: every entry is a hash slot met by
 // some frames of the batch; its block's 512 voxels are held in registers (4
 // per thread) across those frames, in batch order, and written back once.
-// Entries are handed out dynamically (blocks differ in their frame counts);
-// next[g] is double-buffered so one group barrier per entry suffices.  The
-// last CTA to finish resets every map's work list for the next batch.
-template <int NF, int NM, int G, bool COHERENT, int STORAGE, bool PINHOLE_ONLY, bool WEIGHTED, bool FAST>
-__device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, IntegSmem<NF, NM, G>& sm) {
-  static_assert(G == 1 || G == 2, "one or two worker groups per CTA");
-  const int g = G == 1 ? 0 : (int)threadIdx.x / kIntegrateThreads;
-  const int t = G == 1 ? (int)threadIdx.x : (int)threadIdx.x % kIntegrateThreads;
+//
+// A block is four slabs of 128 voxels, one per warp, and warps take slabs by
+// ticket: four consecutive tickets are one entry, so a block's slabs run on
+// one SM at about the same time (their depth gathers share L1 lines), and no
+// warp waits for another to finish a block (a CTA barrier per entry cost 16 %
+// of the warps' time).  The warp that takes an entry's first slab fetches the
+// next entry (handed out dynamically: blocks differ in their frame counts)
+// into a ring of kRing slots; a slot is free once the four slabs of its last
+// entry are done.  Tickets go out in order and an entry's slabs depend on no
+// later one, so both waits end; they are bounded all the same.  The warp that
+// finishes an entry's last slab clears its mask (every slab has read it by
+// then).  The last CTA to finish resets every map's work list.
+template <int NF, int NM, bool COHERENT, int STORAGE, bool PINHOLE_ONLY, bool WEIGHTED, bool FAST>
+__device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, IntegSmem<NF, NM>& sm) {
   if (threadIdx.x < NM) sm.upd[threadIdx.x] = sm.pairs[threadIdx.x] = 0ull;
-  for (int f = threadIdx.x; f < p.n_frames; f += G * kIntegrateThreads)
+  for (int f = threadIdx.x; f < p.n_frames; f += blockDim.x)
     if (p.fr[f].kind == kSensorPinhole) stage_frame(p.fr[f], sm.fp[f]);
-  if (t == 0) sm.next[g][0] = blockIdx.x * G + g;
+  if (threadIdx.x < kRing) {
+    sm.seq[threadIdx.x] = threadIdx.x ? 0xFFFFFFFFu : 0u;
+    sm.entry[threadIdx.x] = blockIdx.x;
+    sm.done[threadIdx.x] = 0u;
+  }
   if (threadIdx.x == 0) {
+    sm.ticket = 0u;
     // the batch's work = the concatenation of every map's list
     uint32_t acc = 0;
     for (int k = 0; k < p.n_maps; ++k) {
@@ -1326,42 +1360,68 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
   }
   __syncthreads();
   const uint32_t n = sm.begin[p.n_maps];
-  // this thread's voxels: x = lx0 .. lx0 + 3 at (ly, lz)
-  const int lx0 = (t & 1) * 4, ly = (t >> 1) & 7, lz = t >> 4;
+  const int lane = threadIdx.x & 31;
 
-  for (uint32_t it = 0;; ++it) {
-    const uint32_t e = sm.next[g][it & 1u];
-    if (e >= n) break;
-    if (t == 0) sm.next[g][(it + 1) & 1u] = gridDim.x * G + atomicAdd(p.maps[0].ctl + 2, 1u);
-    // every thread reads the entry's metadata itself (same addresses across
-    // the group), so no warp waits on another before its voxel loads
-    int mi = 0;
-    while (mi + 1 < p.n_maps && e >= sm.begin[mi + 1]) ++mi;
-    const MapDev& m = NM == 1 ? p.maps[0] : p.maps[mi];
-    const uint32_t slot = meta_load<COHERENT>(m.list + (e - sm.begin[mi]));
-    const int val = meta_load<COHERENT>(m.vals + slot);
-    const uint32_t slot_mask = meta_load<COHERENT>(m.mask + slot);
-    const unsigned long long slot_key = meta_load<COHERENT>(m.keys + slot);
-    const bool fresh = val <= -2;
-    const int pool = fresh ? -val - 2 : val;
-    unsigned long long my_upd = 0;
-    if (val != -1) {
-      float D[4], W[4], G4[4], B[4];
-      if (fresh) {
+  for (;;) {
+    uint32_t k = 0, e = 0;
+    bool ok = true;
+    if (lane == 0) {
+      k = atomicAdd(&sm.ticket, 1u);
+      ok = poll_shared(&sm.seq[(k >> 2) % kRing], k >> 2);
+      e = *(const volatile uint32_t*)&sm.entry[(k >> 2) % kRing];
+    }
+    k = __shfl_sync(0xffffffffu, k, 0);
+    e = __shfl_sync(0xffffffffu, e, 0);
+    const uint32_t seq = k >> 2, next = seq + 1;
+    // the next entry, asked for now and published once this one's voxels are requested
+    uint32_t fetched = e;
+    if ((k & 3u) == 0u && lane == 0 && e < n) fetched = gridDim.x + atomicAdd(p.maps[0].ctl + 2, 1u);
+    int mi = 0, pool = -1;
+    uint32_t slot = 0, bits = 0;
+    float D[4], W[4], G4[4], B[4];
+    VoxelQuad vq;
+    const bool work = e < n && __all_sync(0xffffffffu, ok);
+    // this thread's voxels: x = 2 (lane & 3) and the next, y = lane >> 2, z = 2 slab and the next
+    vq.at = (int)(k & 3u) * 64 + lane;
+    if (work) {
+      if (NM > 1)
+        while (mi + 1 < p.n_maps && e >= sm.begin[mi + 1]) ++mi;
+      const MapDev& m = NM == 1 ? p.maps[0] : p.maps[mi];
+      slot = meta_load<COHERENT>(m.list + (e - sm.begin[mi]));
+      const int val = meta_load<COHERENT>(m.vals + slot);
+      bits = meta_load<COHERENT>(m.mask + slot);
+      const unsigned long long slot_key = meta_load<COHERENT>(m.keys + slot);
+      pool = val <= -2 ? -val - 2 : val;
+      if (val < 0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) { D[i] = 0.0f; W[i] = 0.0f; G4[i] = 0.0f; B[i] = 0.0f; }
       } else {
-        Voxels4<STORAGE>::load(m, pool, t, D, W, G4, B);
+        Voxels4<STORAGE>::load(m, pool, vq.at, D, W, G4, B);
       }
-      const int bx = key_coord(slot_key, 0), by = key_coord(slot_key, 1), bz = key_coord(slot_key, 2);
-      const VoxelRow vr{bx, by, bz, lx0, ly, lz};
-      uint32_t bits = slot_mask;
+      vq.x = (float)(key_coord(slot_key, 0) * 8 + 2 * (lane & 3));
+      vq.y = (float)(key_coord(slot_key, 1) * 8 + (lane >> 2));
+      vq.z = (float)(key_coord(slot_key, 2) * 8 + 2 * (int)(k & 3u));
+    }
+    if ((k & 3u) == 0u && lane == 0) {
+      if (!poll_shared(&sm.done[next % kRing], 4u * (next / kRing))) ok = false;
+      sm.entry[next % kRing] = fetched;
+      __threadfence_block();
+      *(volatile uint32_t*)&sm.seq[next % kRing] = next;
+    }
+    if (!__all_sync(0xffffffffu, ok)) {
+      if (lane == 0) atomicOr(p.maps[0].counters + kCntStatus, (unsigned long long)kStTimeout);
+      break;
+    }
+    if (!work) break;
+    const MapDev& m = NM == 1 ? p.maps[0] : p.maps[mi];
+    uint32_t my_upd = 0;
+    if (pool >= 0) {
       while (bits) {
         // bit k of the mask is frame k of the batch; frames apply in batch
         // order.  Two consecutive pinhole frames issue all their depth loads
         // before the first update (longer runs measured slower: the unrolled
         // code outgrows the instruction cache).
-        int fq[4];
+        int fq[2];
         int nq = 0;
         bool go = true;
 #pragma unroll
@@ -1378,28 +1438,31 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
             }
           }
         }
-        fq[2] = fq[3] = -1;
         if (nq == 2)
-          fuse_pinhole<2, STORAGE, WEIGHTED, FAST, PINHOLE_ONLY>(p, sm.fp, fq, m, vr, D, W, G4, B, my_upd);
+          fuse_pinhole<2, STORAGE, WEIGHTED, FAST>(p, sm.fp, fq, m, vq, D, W, G4, B, my_upd);
         else if (nq == 1)
-          fuse_pinhole<1, STORAGE, WEIGHTED, FAST, PINHOLE_ONLY>(p, sm.fp, fq, m, vr, D, W, G4, B, my_upd);
+          fuse_pinhole<1, STORAGE, WEIGHTED, FAST>(p, sm.fp, fq, m, vq, D, W, G4, B, my_upd);
         else if (!PINHOLE_ONLY) {
           const int f = __ffs(bits) - 1;  // a LiDAR frame
           bits &= bits - 1u;
-          fuse_lidar<STORAGE, WEIGHTED>(p.fr[f], m, vr, D, W, my_upd);
+          fuse_lidar<STORAGE, WEIGHTED>(p.fr[f], m, vq, D, W, my_upd);
         }
       }
-      Voxels4<STORAGE>::store(m, pool, t, D, W, G4, B);
+      Voxels4<STORAGE>::store(m, pool, vq.at, D, W, G4, B);
     }
-    // per-map update count: warp sums into a shared per-map counter
-    for (int o = 16; o > 0; o >>= 1) my_upd += __shfl_down_sync(0xffffffffu, my_upd, o);
-    if ((t & 31) == 0 && my_upd) atomicAdd(&sm.upd[mi], my_upd);
-    group_sync<G>(g);  // every warp of the group has read this entry's metadata
-    if (t == 0) {
-      atomicAdd(&sm.pairs[mi], (unsigned long long)__popc(slot_mask));
-      m.mask[slot] = 0u;
-      if (fresh) m.vals[slot] = pool;
-      if (m.dirty && val != -1) m.dirty[pool] = kDirtyEsdf | kDirtyMesh;
+    // per-map update count; the entry's last slab clears its metadata
+    my_upd = __reduce_add_sync(0xffffffffu, my_upd);
+    if (lane == 0) {
+      if (my_upd) atomicAdd(&sm.upd[mi], (unsigned long long)my_upd);
+      __threadfence_block();
+      if (atomicAdd(&sm.done[seq % kRing], 1u) == 4u * (seq / kRing) + 3u) {
+        atomicAdd(&sm.pairs[mi], (unsigned long long)__popc(meta_load<COHERENT>(m.mask + slot)));
+        m.mask[slot] = 0u;
+        if (pool >= 0) {
+          m.vals[slot] = pool;  // no longer new
+          if (m.dirty) m.dirty[pool] = kDirtyEsdf | kDirtyMesh;
+        }
+      }
     }
   }
   if (p.overlap) allow_next_grid();
@@ -1426,11 +1489,11 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
 }
 
 template <int NF, int NM, int STORAGE, bool PINHOLE_ONLY, bool WEIGHTED, bool FAST = false>
-__global__ void __launch_bounds__(kIntegrateThreads)
+__global__ void __launch_bounds__(kIntegrateThreads, STORAGE == kStorageColor ? 6 : 7)
     integrate_kernel(const __grid_constant__ BatchParams<NF, NM> p) {
-  __shared__ IntegSmem<NF, NM, 1> sm;
+  __shared__ IntegSmem<NF, NM> sm;
   if (p.overlap) wait_prev_grid();
-  integrate_entries<NF, NM, 1, false, STORAGE, PINHOLE_ONLY, WEIGHTED, FAST>(p, sm);
+  integrate_entries<NF, NM, false, STORAGE, PINHOLE_ONLY, WEIGHTED, FAST>(p, sm);
 }
 
 // ------------------------------------------- one launch per batch (fused)
@@ -1477,20 +1540,19 @@ __device__ __noinline__ bool grid_wait(unsigned int* count, unsigned int expecte
   return s_ok != 0;
 }
 
-constexpr int kFusedThreads = kAllocThreads;  // two integration worker groups
-static_assert(kFusedThreads == 2 * kIntegrateThreads, "fused CTA = two integration groups");
+constexpr int kFusedThreads = kAllocThreads;
 
 template <int NF, int NM, int TH>
 union FusedSmem {
   AllocSmem<TH> a;
-  IntegSmem<NF, NM, 2> i;
+  IntegSmem<NF, NM> i;
 };
 
 // Allocation and integration of one batch in one persistent, cooperative
 // launch: the CTAs walk every allocation tile of the batch (grid-stride),
 // meet at a bounded grid-wide wait (the integration reads the work list,
 // slot masks and pool indices that every tile wrote), then integrate the
-// work list as two groups of kIntegrateThreads per CTA.  Single-map
+// work list.  Single-map
 // batches, TSDF storage, constant weighting, no walk statistics.
 // Four resident CTAs per SM (64 registers): the rig's fused step measured
 // 16.1 ms per 1,000 frames against 18.2 ms with three.
@@ -1502,7 +1564,8 @@ __global__ void __launch_bounds__(kFusedThreads, 4)
     alloc_tile<NF, NM, TH, PINHOLE_ONLY, false, FAST, true>(p, tile_frame(p, cta), cta, sm.a);
   if (!grid_wait(p.maps[0].ctl + 3, gridDim.x + (unsigned)p.wait_extra, p.maps[0].counters + kCntStatus))
     return;  // timed out: integration skipped, the map reports TSDF_ERR_TIMEOUT
-  integrate_entries<NF, NM, 2, true, STORAGE, PINHOLE_ONLY, false, FAST>(p, sm.i);
+  __syncthreads();  // the tiles' shared memory is free for the integration
+  integrate_entries<NF, NM, true, STORAGE, PINHOLE_ONLY, false, FAST>(p, sm.i);
 }
 
 template <int STORAGE>
@@ -1601,11 +1664,11 @@ __global__ void decay_kernel(const MapDev m, float d_occ, float d_free) {
   }
 }
 
-// Empty a map: hash slots, both mask sets, changed flags, counters and
+// Empty a map: hash slots, every mask set, changed flags, counters and
 // control words in one launch, four slots or 16 flags per thread and step in
 // 16-byte stores.  One kernel and three memsets before cost a step over 16
 // maps four launches a map (85 us of its 1,040 us).
-__global__ void reset_kernel(const MapDev m, uint32_t cap, uint32_t* mask1, unsigned int* ctl1) {
+__global__ void reset_kernel(const MapDev m, uint32_t cap, const MoreSets more) {
   const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
   const uint4 ones = make_uint4(~0u, ~0u, ~0u, ~0u), zero = make_uint4(0u, 0u, 0u, 0u);
   static_assert(kEmptyKey == ~0ull, "an empty key is all ones");
@@ -1614,18 +1677,23 @@ __global__ void reset_kernel(const MapDev m, uint32_t cap, uint32_t* mask1, unsi
     reinterpret_cast<uint4*>(m.keys)[2 * i + 1] = ones;
     reinterpret_cast<uint4*>(m.vals)[i] = ones;  // -1 each
     reinterpret_cast<uint4*>(m.mask)[i] = zero;
-    reinterpret_cast<uint4*>(mask1)[i] = zero;
+#pragma unroll
+    for (int k = 0; k < kSets - 1; ++k) reinterpret_cast<uint4*>(more.mask[k])[i] = zero;
   }
   for (uint32_t i = cap / 4 * 4 + first; i < cap; i += step) {  // a table of two slots
     m.keys[i] = kEmptyKey;
     m.vals[i] = -1;
-    m.mask[i] = mask1[i] = 0u;
+    m.mask[i] = 0u;
+    for (int k = 0; k < kSets - 1; ++k) more.mask[k][i] = 0u;
   }
   const uint32_t nd = (uint32_t)m.max_blocks;
   for (uint32_t i = first; i < nd / 16; i += step) reinterpret_cast<uint4*>(m.dirty)[i] = zero;
   for (uint32_t i = nd / 16 * 16 + first; i < nd; i += step) m.dirty[i] = 0;
   if (first < kNumCounters) m.counters[first] = 0ull;
-  if (first < 4) m.ctl[first] = ctl1[first] = 0u;
+  if (first < 4) {
+    m.ctl[first] = 0u;
+    for (int k = 0; k < kSets - 1; ++k) more.ctl[k][first] = 0u;
+  }
 }
 
 }  // namespace
@@ -1716,8 +1784,43 @@ cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, AllocSha
               : launch_k(band_alloc_kernel<NF, NM, kTileHSmall, false, false, false, false>, g, b, s, p);
 }
 
+// Launch integration kernel k on a persistent grid: per_sm CTAs per SM (the
+// map's knob), or if that is 0 as many as can be resident with this variant's
+// registers, at most `limit` (0: no limit).  Batches of many pinhole frames
+// are limited: an entry is then long work (up to 32 frames), and with every
+// SM full of entries half of them are started at once and the chip drains
+// unevenly (32 frames of 640x480, us per launch with 3, 4, 5, 7 and 9 CTAs per SM:
+// 56.6, 55.1, 55.3, 61.8, 61.4).  Single frames and LiDAR scans want every warp
+// (a scan with 4, 5, 7: 53, 47, 43).
+constexpr int kManyFrames = 8, kManyFramesPerSm = 5;
+template <class P>
+cudaError_t launch_persistent(void (*k)(P), int per_sm, int limit, cudaStream_t s, const P& p,
+                              std::atomic<int>& fit) {
+  int n = fit.load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kIntegrateThreads, 0) != cudaSuccess || n <= 0) {
+      cudaGetLastError();
+      n = 4;
+    }
+    fit.store(n, std::memory_order_relaxed);
+  }
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return cudaGetLastError();
+  if (per_sm > 0) n = std::min(n, per_sm);
+  else if (limit > 0) n = std::min(n, limit);
+  return launch_k(k, dim3(std::max(1, sms) * n), dim3(kIntegrateThreads), s, p);
+}
+
+template <int NF, int NM, int STORAGE, bool PINHOLE_ONLY, bool WEIGHTED, bool FAST>
+cudaError_t launch_variant(const BatchParams<NF, NM>& p, int per_sm, int limit, cudaStream_t s) {
+  static std::atomic<int> fit{0};  // resident CTAs per SM of this variant (all devices are alike here)
+  return launch_persistent(integrate_kernel<NF, NM, STORAGE, PINHOLE_ONLY, WEIGHTED, FAST>, per_sm, limit, s, p, fit);
+}
+
 template <int NF, int NM>
-cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int n_ctas, cudaStream_t s) {
+cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int per_sm, cudaStream_t s) {
   // all maps of a batch share one storage type (checked by the host API)
   // colour maps take pinhole frames only (checked by the host API)
   const bool ph = pinhole_only(p);
@@ -1726,25 +1829,27 @@ cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int n_ctas, cudaStrea
   // one weighted map selects the weighted kernel for the whole batch
   bool wt = false;
   for (int k = 0; k < p.n_maps; ++k) wt = wt || p.maps[k].weighting != 0;
-  const dim3 g(n_ctas), b(kIntegrateThreads);
   // FAST: pinhole reciprocals by rcp_dec<true> (the host checked their range)
   const bool fast = p.fast_rcp != 0;
+  const int limit = ph && st != kStorageColor && p.n_frames >= kManyFrames ? kManyFramesPerSm : 0;
 #define GBT_INTEG(ST, PH) \
-  (fast ? launch_k(integrate_kernel<NF, NM, ST, PH, false, true>, g, b, s, p) \
-        : launch_k(integrate_kernel<NF, NM, ST, PH, false, false>, g, b, s, p))
+  (fast ? launch_variant<NF, NM, ST, PH, false, true>(p, per_sm, limit, s) \
+        : launch_variant<NF, NM, ST, PH, false, false>(p, per_sm, limit, s))
+#define GBT_WEIGHTED(ST) launch_variant<NF, NM, ST, false, true, false>(p, per_sm, limit, s)
   if (st == kStorageColor) return GBT_INTEG(kStorageColor, true);
   if (st == kStorageOcc) return ph ? GBT_INTEG(kStorageOcc, true) : GBT_INTEG(kStorageOcc, false);
   if (st == kStorageX16) {
-    if (wt) return launch_k(integrate_kernel<NF, NM, kStorageX16, false, true>, g, b, s, p);
+    if (wt) return GBT_WEIGHTED(kStorageX16);
     return ph ? GBT_INTEG(kStorageX16, true) : GBT_INTEG(kStorageX16, false);
   }
   if (st == kStorageF16) {
-    if (wt) return launch_k(integrate_kernel<NF, NM, kStorageF16, false, true>, g, b, s, p);
+    if (wt) return GBT_WEIGHTED(kStorageF16);
     return ph ? GBT_INTEG(kStorageF16, true) : GBT_INTEG(kStorageF16, false);
   }
-  if (wt) return launch_k(integrate_kernel<NF, NM, kStorageF32, false, true>, g, b, s, p);
+  if (wt) return GBT_WEIGHTED(kStorageF32);
   return ph ? GBT_INTEG(kStorageF32, true) : GBT_INTEG(kStorageF32, false);
 #undef GBT_INTEG
+#undef GBT_WEIGHTED
 }
 
 // The fused kernel of a tile height for a storage and sensor mix, launched
@@ -1849,48 +1954,13 @@ cudaError_t launch_decay(const MapDev& m, float d_occ, float d_free, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_reset(const MapDev& m, uint32_t cap, uint32_t* mask1, unsigned int* ctl1, cudaStream_t s) {
+cudaError_t launch_reset(const MapDev& m, uint32_t cap, const MoreSets& more, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const unsigned need = std::max((cap / 4 + 255) / 256, ((unsigned)m.max_blocks / 16 + 255) / 256);
-  reset_kernel<<<std::max(1u, std::min(need, (unsigned)sms * 8)), 256, 0, s>>>(m, cap, mask1, ctl1);
+  reset_kernel<<<std::max(1u, std::min(need, (unsigned)sms * 8)), 256, 0, s>>>(m, cap, more);
   return cudaGetLastError();
-}
-
-namespace {
-template <class K>
-int occupancy(K kernel) {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kIntegrateThreads, 0) != cudaSuccess)
-    n = 0;
-  return n;
-}
-}  // namespace
-
-// Resident integration CTAs per SM: the smallest over the kernel variants a
-// map of this storage can launch (the grid is persistent).
-int integrate_ctas_per_sm(int storage) {
-  constexpr int F = kMaxFrames, M = kMaxMaps;
-  int n;
-  if (storage == kStorageColor)
-    n = occupancy(integrate_kernel<F, M, kStorageColor, true, false>);
-  else if (storage == kStorageOcc)
-    n = std::min(occupancy(integrate_kernel<F, M, kStorageOcc, true, false>),
-                 occupancy(integrate_kernel<F, M, kStorageOcc, false, false>));
-  else if (storage == kStorageX16)
-    n = std::min({occupancy(integrate_kernel<F, M, kStorageX16, true, false>),
-                  occupancy(integrate_kernel<F, M, kStorageX16, false, false>),
-                  occupancy(integrate_kernel<F, M, kStorageX16, false, true>)});
-  else if (storage == kStorageF16)
-    n = std::min({occupancy(integrate_kernel<F, M, kStorageF16, true, false>),
-                  occupancy(integrate_kernel<F, M, kStorageF16, false, false>),
-                  occupancy(integrate_kernel<F, M, kStorageF16, false, true>)});
-  else
-    n = std::min({occupancy(integrate_kernel<F, M, kStorageF32, true, false>),
-                  occupancy(integrate_kernel<F, M, kStorageF32, false, false>),
-                  occupancy(integrate_kernel<F, M, kStorageF32, false, true>)});
-  return n > 0 ? n : 4;
 }
 
 }  // namespace gbt

@@ -37,18 +37,16 @@ struct tsdf_map {
   float v, wmax;
   int32_t trunc;
   double vd, Bd;
-  int n_ctas_integrate;
+  int integrate_per_sm;  // integration CTAs per SM, 0 = as many as fit
   int tile_h;  // allocation tile height, 0 = automatic
   int launch_mode;     // TSDF_LAUNCH_SPLIT or TSDF_LAUNCH_FUSED
   int32_t wait_extra;  // map_wait_test: extra CTAs the fused launch's grid-wide wait expects
   int64_t frames;
   unsigned long long status_seen;  // device status bits observed by the host
   std::vector<LidarTable> tables;
-  // second mask / work-list / control set: with it the allocation of one
-  // sub-batch runs on `aux` while the previous sub-batch integrates
-  uint32_t* mask1;
-  uint32_t* list1;
-  unsigned int* ctl1;
+  // further mask / work-list / control sets: with them the allocation of
+  // sub-batches runs on `aux` while earlier ones integrate
+  gbt::MoreSets more;
   cudaStream_t aux;
   cudaEvent_t ev_alloc[4], ev_int[4], ev_start;
   // host-input batches: copy stream and per-sub-batch copy events (lazy)
@@ -72,6 +70,7 @@ struct tsdf_map {
 
 namespace {
 
+static_assert(gbt::kSets <= 4, "one of the four integration events per set");
 constexpr int64_t kDefaultBlocks = 1 << 18;
 constexpr size_t kTimedCalls = 4096;
 constexpr int32_t kMaxBatchFrames = 1 << 16;
@@ -213,6 +212,7 @@ bool fast_rcp_ok(const FrameDev& F, double v, int lidar_lsb) {
     int L2 = lsb_rc == INT_MAX ? INT_MAX : lsb_rc + lsb_exp(half_v);
     if (F.tloc[2] != 0.0f) L2 = std::min(L2, lsb_exp(F.tloc[2]));
     const double max_q = (16777216.0 + 16.0) * (double)(float)v * (1.0 + 1e-6);  // |rel| < 2^24 + 8
+    if (F.width > (1 << 22) || F.height > (1 << 22)) return false;  // the kernels' floor of pixel coordinates
     if (L2 < -126 || 3.0 * max_rc * max_q + std::fabs((double)F.tloc[2]) >= kTwo126) return false;
     return true;
   }
@@ -370,13 +370,13 @@ cudaEvent_t* timing_slot(tsdf_map* m) {
   return &m->events[4 * m->n_timed++];
 }
 
-// Device view of map m using mask / list / control set `set` (0 or 1).
+// Device view of map m using mask / list / control set `set` (0 .. kSets - 1).
 MapDev view_set(const tsdf_map* m, int set) {
   MapDev d = m->dev;
   if (set) {
-    d.mask = m->mask1;
-    d.list = m->list1;
-    d.ctl = m->ctl1;
+    d.mask = m->more.mask[set - 1];
+    d.list = m->more.list[set - 1];
+    d.ctl = m->more.ctl[set - 1];
   }
   return d;
 }
@@ -408,7 +408,7 @@ tsdf_status integrate_one(tsdf_map* m, int kind, const tsdf_pinhole* ph, const t
     cudaEventRecord(ev[1], s);
     cudaEventRecord(ev[2], s);
   }
-  if (gbt::launch_integrate(p, m->n_ctas_integrate, s) != cudaSuccess) return cuda_fail();
+  if (gbt::launch_integrate(p, m->integrate_per_sm, s) != cudaSuccess) return cuda_fail();
   if (ev) cudaEventRecord(ev[3], s);
   m->frames += 1;
   return TSDF_OK;
@@ -424,9 +424,11 @@ tsdf_status read_counters(const tsdf_map* m, unsigned long long c[gbt::kNumCount
 }
 
 void free_map(tsdf_map* m) {
-  cudaFree(m->mask1);
-  cudaFree(m->list1);
-  cudaFree(m->ctl1);
+  for (int k = 0; k < gbt::kSets - 1; ++k) {
+    cudaFree(m->more.mask[k]);
+    cudaFree(m->more.list[k]);
+    cudaFree(m->more.ctl[k]);
+  }
   cudaFree(m->dev.dirty);
   if (m->mesh_on) {
     cudaFree(m->mesh.list);
@@ -520,6 +522,7 @@ tsdf_status map_create_ex(float voxel_size, int32_t truncation_voxels, float max
 
   tsdf_map* m = new tsdf_map();
   std::memset(&m->dev, 0, sizeof(m->dev));
+  std::memset(&m->more, 0, sizeof(m->more));
   if (cudaGetDevice(&m->device) != cudaSuccess) {
     delete m;
     return cuda_fail();
@@ -563,27 +566,24 @@ tsdf_status map_create_ex(float voxel_size, int32_t truncation_voxels, float max
             cudaMalloc(&d.counters, sizeof(unsigned long long) * gbt::kNumCounters) == cudaSuccess &&
             cudaMalloc(&d.list, sizeof(uint32_t) * o.max_blocks) == cudaSuccess &&
             cudaMalloc(&d.ctl, sizeof(unsigned int) * 4) == cudaSuccess &&
-            cudaMalloc(&m->mask1, sizeof(uint32_t) * cap) == cudaSuccess &&
-            cudaMalloc(&m->list1, sizeof(uint32_t) * o.max_blocks) == cudaSuccess &&
-            cudaMalloc(&m->ctl1, sizeof(unsigned int) * 4) == cudaSuccess &&
             cudaMalloc(&d.dirty, (size_t)o.max_blocks) == cudaSuccess &&
             cudaStreamCreateWithFlags(&m->aux, cudaStreamNonBlocking) == cudaSuccess &&
             cudaEventCreateWithFlags(&m->ev_start, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; ok && i < 4; ++i)
     ok = cudaEventCreateWithFlags(&m->ev_alloc[i], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&m->ev_int[i], cudaEventDisableTiming) == cudaSuccess;
+  for (int k = 0; ok && k < gbt::kSets - 1; ++k)
+    ok = cudaMalloc(&m->more.mask[k], sizeof(uint32_t) * cap) == cudaSuccess &&
+         cudaMalloc(&m->more.list[k], sizeof(uint32_t) * o.max_blocks) == cudaSuccess &&
+         cudaMalloc(&m->more.ctl[k], sizeof(unsigned int) * 4) == cudaSuccess;
   if (ok)
-    ok = gbt::launch_reset(d, m->cap, m->mask1, m->ctl1, 0) == cudaSuccess &&
+    ok = gbt::launch_reset(d, m->cap, m->more, 0) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;
   if (!ok) {
     free_map(m);
     return cuda_fail();
   }
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
-  int per_sm = gbt::integrate_ctas_per_sm(o.storage);
-  if (o.integrate_ctas_per_sm > 0) per_sm = std::min(per_sm, o.integrate_ctas_per_sm);
-  m->n_ctas_integrate = std::max(1, sms) * per_sm;
+  m->integrate_per_sm = o.integrate_ctas_per_sm;
   m->tile_h = o.alloc_tile_h;
   m->launch_mode = o.launch_mode;
   m->wait_extra = 0;
@@ -652,9 +652,9 @@ using SubBatchHook = tsdf_status (*)(void* ctx, int b, int f0, int nf, cudaStrea
 
 // Sub-batches of up to 32 frames, each one allocation launch and one
 // integration launch.  With more than one, sub-batch b uses mask / list set
-// b % 2 and its allocation runs on the lead map's auxiliary stream,
-// overlapping the integration of sub-batch b - 1 on the caller's stream; it
-// waits for the integration of b - 2, which used the same set.
+// b % kSets and its allocation runs on the lead map's auxiliary stream,
+// overlapping the integration of earlier sub-batches on the caller's stream;
+// it waits for the integration of b - kSets, which used the same set.
 tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDev>& fr, int32_t n,
                       cudaStream_t s, SubBatchHook hook, void* ctx) {
   // the params block is large; keep it off the stack
@@ -699,7 +699,7 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
           cudaEventRecord(ev[1], s);
           cudaEventRecord(ev[2], s);
         }
-        if (gbt::launch_integrate(p1, lead->n_ctas_integrate, s) != cudaSuccess) return cuda_fail();
+        if (gbt::launch_integrate(p1, lead->integrate_per_sm, s) != cudaSuccess) return cuda_fail();
         if (ev) cudaEventRecord(ev[3], s);
         if (cudaEventRecord(lead->ev_int[b & 3], s) != cudaSuccess) return cuda_fail();
         continue;
@@ -722,7 +722,8 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
   for (int b = 0; b < n_sub; ++b) {
     const int f0 = b * gbt::kMaxFrames, nf = std::min(gbt::kMaxFrames, n - f0);
     cudaStream_t sa = piped ? lead->aux : s;
-    if (piped && b >= 2 && cudaStreamWaitEvent(sa, lead->ev_int[(b - 2) & 3], 0) != cudaSuccess)
+    if (piped && b >= gbt::kSets &&
+        cudaStreamWaitEvent(sa, lead->ev_int[(b - gbt::kSets) & 3], 0) != cudaSuccess)
       return cuda_fail();
     if (hook) {
       tsdf_status st = hook(ctx, b, f0, nf, sa);
@@ -731,7 +732,7 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
     std::memset(&p, 0, sizeof(p));
     p.n_frames = nf;
     p.n_maps = n_maps;
-    for (int i = 0; i < n_maps; ++i) p.maps[i] = view_set(maps[i], piped ? (b & 1) : 0);
+    for (int i = 0; i < n_maps; ++i) p.maps[i] = view_set(maps[i], piped ? b % gbt::kSets : 0);
     p.fast_rcp = 1;
     for (int f = 0; f < nf; ++f) {
       p.fr[f] = fr[f0 + f];
@@ -760,8 +761,8 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
                   cudaStreamWaitEvent(s, lead->ev_alloc[b & 3], 0) != cudaSuccess))
       return cuda_fail();
     if (ev) cudaEventRecord(ev[2], s);
-    if ((n_maps == 1 ? gbt::launch_integrate(p1, lead->n_ctas_integrate, s)
-                     : gbt::launch_integrate(p, lead->n_ctas_integrate, s)) != cudaSuccess)
+    if ((n_maps == 1 ? gbt::launch_integrate(p1, lead->integrate_per_sm, s)
+                     : gbt::launch_integrate(p, lead->integrate_per_sm, s)) != cudaSuccess)
       return cuda_fail();
     if (ev) cudaEventRecord(ev[3], s);
     if (piped && cudaEventRecord(lead->ev_int[b & 3], s) != cudaSuccess) return cuda_fail();
@@ -1379,7 +1380,7 @@ tsdf_status map_reset(tsdf_map* map, void* cuda_stream) {
   if (!on_device(map)) return TSDF_ERR_STATE;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   if (map->esdf_on && gbt::launch_esdf_reset(map->dev, map->esdf, s) != cudaSuccess) return cuda_fail();
-  if (gbt::launch_reset(map->dev, map->cap, map->mask1, map->ctl1, s) != cudaSuccess) return cuda_fail();
+  if (gbt::launch_reset(map->dev, map->cap, map->more, s) != cudaSuccess) return cuda_fail();
   map->status_seen = 0;
   map->frames = 0;
   return TSDF_OK;
@@ -1507,10 +1508,6 @@ tsdf_status integrate_depth_static(const tsdf_map_buffers* buf, float voxel_size
   F.fast_rcp = p.fast_rcp = fast_rcp_ok(F, (double)voxel_size, INT_MAX) ? 1 : 0;
   F.short_walks = short_walks_ok(F, truncation_voxels) ? 1 : 0;
 
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return cuda_fail();
   cudaStream_t s = (cudaStream_t)cuda_stream;
   // the control words must start at zero; a previous call leaves them so,
   // but a call that never ran to completion might not have
@@ -1518,9 +1515,7 @@ tsdf_status integrate_depth_static(const tsdf_map_buffers* buf, float voxel_size
   const gbt::AllocShape shape = gbt::pick_alloc_shape(p, 0);
   const int ctas = number_tiles(p, shape);
   if (gbt::launch_band_alloc(p, ctas, shape, s) != cudaSuccess) return cuda_fail();
-  if (gbt::launch_integrate(p, std::max(1, sms) * gbt::integrate_ctas_per_sm(TSDF_STORAGE_FP32), s) !=
-      cudaSuccess)
-    return cuda_fail();
+  if (gbt::launch_integrate(p, 0, s) != cudaSuccess) return cuda_fail();
   return TSDF_OK;
 }
 

@@ -103,6 +103,15 @@ struct MapDev {
   uint8_t* dirty;                 // [max_blocks] kDirtyEsdf / kDirtyMesh: changed since the
                                   // last ESDF update / mesh extraction (may be null)
 };
+// A map has kSets mask / work-list / control sets: the allocation of up to
+// kSets - 1 sub-batches can run ahead of the integration.  The first is
+// MapDev's own.
+constexpr int kSets = 2;
+struct MoreSets {
+  uint32_t* mask[kSets - 1];
+  uint32_t* list[kSets - 1];
+  unsigned int* ctl[kSets - 1];
+};
 // kDirtyNbr: a face neighbour changed (occupancy ESDF sites read across faces)
 enum : uint8_t { kDirtyEsdf = 1, kDirtyMesh = 2, kDirtyNbr = 4 };
 
@@ -315,7 +324,7 @@ AllocShape pick_alloc_shape(const BatchParams<NF, NM>& p, int tile_h);
 template <int NF, int NM>
 cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, AllocShape shape, cudaStream_t s);
 template <int NF, int NM>
-cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int n_ctas, cudaStream_t s);
+cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int per_sm, cudaStream_t s);
 // Allocation and integration of one batch in a single cooperative launch;
 // cudaErrorNotSupported for batches it does not cover (the caller then
 // launches the two kernels).
@@ -338,7 +347,7 @@ cudaError_t launch_query_color(const MapDev& m, const float* pts, int64_t n, flo
                                cudaStream_t s);
 cudaError_t launch_query(const MapDev& m, const float* pts, int64_t n, float* dist, float* weight,
                          cudaStream_t s);
-cudaError_t launch_reset(const MapDev& m, uint32_t cap, uint32_t* mask1, unsigned int* ctl1, cudaStream_t s);
+cudaError_t launch_reset(const MapDev& m, uint32_t cap, const MoreSets& more, cudaStream_t s);
 cudaError_t launch_decay(const MapDev& m, float d_occ, float d_free, cudaStream_t s);
 // Forget the ESDF states of the map's blocks; before launch_reset, which
 // forgets how many there are.
@@ -367,6 +376,5 @@ struct MeshDev {
 cudaError_t launch_mesh(const MapDev& m, const MeshDev& md, const MeshTable& table, int changed_only,
                         uint32_t gen, float min_weight, float* pos, int32_t* keys, int32_t* cubes,
                         int64_t cap, cudaStream_t s);
-int integrate_ctas_per_sm(int storage);
 
 }  // namespace gbt

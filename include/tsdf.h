@@ -387,8 +387,8 @@ typedef struct {
  * a missing block is unknown); site_eps and min_weight are not used; the
  * blocks marked are the changed ones and their face neighbours, and a
  * map_decay_occupancy call counts as a change of every block it alters.
- * Enqueued on cuda_stream; waits for the stream after every four iterations
- * to test for convergence.
+ * Enqueued on cuda_stream; waits for the stream.  TSDF_ERR_TIMEOUT if a
+ * bounded device wait gave up.
  */
 tsdf_status map_esdf_update(tsdf_map* map, const tsdf_esdf_opts* opts, void* cuda_stream);
 

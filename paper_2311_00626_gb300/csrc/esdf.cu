@@ -14,21 +14,20 @@
 //                      across block faces)
 //   esdf_clear_kernel  in every block near one of the latter, drop parents
 //                      that are no longer sites
-//   esdf_nbr_kernel    the face-neighbour table of every block
-//   then, until the update set is empty (the host enqueues four iterations
-//   at a time and reads the set size after them):
-//   esdf_sweep_kernel  six in-block sweeps (+x, -x, +y, -y, +z, -z) of every
-//                      block of the update set, in shared memory; the block
-//                      and its existing face neighbours join the tlist
-//   esdf_pull_kernel   every tlist block tries, on its faces, the parents of
-//                      the adjacent voxels across the faces, reading the
-//                      states as they were before this step; results go to
-//                      st2
-//   esdf_apply_kernel  copy back the blocks that changed; they form the next
-//                      update set
+//   esdf_lower_kernel  one cooperative launch: the face-neighbour table of
+//                      every block, then the lowering iterations until no
+//                      block changes.  An iteration is six in-block sweeps
+//                      (+x, -x, +y, -y, +z, -z) of every block of the update
+//                      set, then an exchange in which the set and its
+//                      existing face neighbours try, on their faces, the
+//                      parents of the adjacent voxels across the faces, all
+//                      reading the states as they were before the exchange;
+//                      the blocks that changed are the next update set.
 //
 // All distance arithmetic is on integer offsets (squared lengths), so the
 // result is exact and does not depend on the order in which CTAs run.
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "tsdf_internal.cuh"
@@ -115,9 +114,9 @@ __device__ __forceinline__ uint32_t marked_state(uint32_t old, bool obs, bool si
 // Update-set and lost-site bookkeeping of a marked block (lane 0).
 __device__ __forceinline__ void mark_done(const MapDev& m, const EsdfDev& e, uint32_t p, uint32_t gen, bool any,
                                           bool lost) {
-  if (any) add_update(e, e.list[0], e.cnt, p, gen);
+  if (any) add_update(e, e.list, e.cnt + kEcUpdate, p, gen);
   if (lost) {
-    e.clist[atomicAdd(e.cnt + 2, 1u)] = p;
+    e.clist[atomicAdd(e.cnt + kEcLost, 1u)] = p;
     const unsigned long long key = m.block_keys[p];
     const int G = parent_reach(e) + 1;
     const int cx = key_coord(key, 0) + kCoordBias, cy = key_coord(key, 1) + kCoordBias,
@@ -280,7 +279,7 @@ __global__ void __launch_bounds__(kEsdfThreads)
 __global__ void __launch_bounds__(kEsdfThreads)
     esdf_clear_kernel(const MapDev m, const EsdfDev e, uint32_t gen) {
   constexpr int kWarps = kEsdfThreads / 32;
-  const uint32_t nc = __ldcg(e.cnt + 2);
+  const uint32_t nc = __ldcg(e.cnt + kEcLost);
   if (nc == 0) return;
   const uint32_t nb = n_blocks(m);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -329,7 +328,7 @@ __global__ void __launch_bounds__(kEsdfThreads)
           any = true;
         }
       }
-    if (__any_sync(0xffffffffu, any) && lane == 0) add_update(e, e.list[0], e.cnt, p, gen);
+    if (__any_sync(0xffffffffu, any) && lane == 0) add_update(e, e.list, e.cnt + kEcUpdate, p, gen);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) my_cleared += __shfl_down_sync(0xffffffffu, my_cleared, o);
@@ -340,7 +339,7 @@ __global__ void __launch_bounds__(kEsdfThreads)
 
 // Face-neighbour table of every pool block (the block set does not change
 // during an update).
-__global__ void esdf_nbr_kernel(const MapDev m, const EsdfDev e) {
+__device__ __forceinline__ void neighbour_table(const MapDev& m, const EsdfDev& e) {
   const uint32_t nb = n_blocks(m);
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < 6u * nb; k += gridDim.x * blockDim.x) {
     const uint32_t p = k / 6u;
@@ -351,6 +350,7 @@ __global__ void esdf_nbr_kernel(const MapDev m, const EsdfDev e) {
                        key_coord(key, 2) + (f >> 1 == 2 ? d : 0));
   }
 }
+__global__ void esdf_nbr_kernel(const MapDev m, const EsdfDev e) { neighbour_table(m, e); }
 
 // In-block sweeps keep the block in shared memory padded to 9 words per
 // x-row and 72 per z-slice, so that the lines of every axis are read with at
@@ -380,142 +380,257 @@ __device__ __forceinline__ void relax_line(uint32_t& ps, int& p2, uint32_t qs, i
   }
 }
 
-// Both sweeps along AXIS of one line of eight voxels (first i = 1 .. 7, each
+// Both sweeps along AXIS of two lines of eight voxels (first i = 1 .. 7, each
 // voxel trying its predecessor's parent, then i = 6 .. 0, each trying its
-// successor's), in registers.
+// successor's), in registers; two lines per lane overlap their chains.
 template <int AXIS>
-__device__ __forceinline__ void sweep_line(uint32_t* s, int* s2, int base, int max2) {
+__device__ __forceinline__ void sweep_lines(uint32_t* s, int* s2, int base0, int base1, int max2) {
   constexpr int stride = AXIS == 0 ? 1 : (AXIS == 1 ? kSweepRow : kSweepSlice);
-  uint32_t w[8];
-  int d2[8];
+  uint32_t w0[8], w1[8];
+  int d0[8], d1[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    w[i] = s[base + stride * i];
-    d2[i] = s2[base + stride * i];
+    w0[i] = s[base0 + stride * i];
+    d0[i] = s2[base0 + stride * i];
+    w1[i] = s[base1 + stride * i];
+    d1[i] = s2[base1 + stride * i];
   }
 #pragma unroll
-  for (int i = 1; i < 8; ++i) relax_line<AXIS, -1>(w[i], d2[i], w[i - 1], d2[i - 1], max2);
+  for (int i = 1; i < 8; ++i) {
+    relax_line<AXIS, -1>(w0[i], d0[i], w0[i - 1], d0[i - 1], max2);
+    relax_line<AXIS, -1>(w1[i], d1[i], w1[i - 1], d1[i - 1], max2);
+  }
 #pragma unroll
-  for (int i = 6; i >= 0; --i) relax_line<AXIS, 1>(w[i], d2[i], w[i + 1], d2[i + 1], max2);
+  for (int i = 6; i >= 0; --i) {
+    relax_line<AXIS, 1>(w0[i], d0[i], w0[i + 1], d0[i + 1], max2);
+    relax_line<AXIS, 1>(w1[i], d1[i], w1[i + 1], d1[i + 1], max2);
+  }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    s[base + stride * i] = w[i];
-    s2[base + stride * i] = d2[i];
+    s[base0 + stride * i] = w0[i];
+    s2[base0 + stride * i] = d0[i];
+    s[base1 + stride * i] = w1[i];
+    s2[base1 + stride * i] = d1[i];
   }
 }
 
-// Six in-block sweeps of every block of the current update set (+x, -x,
-// +y, -y, +z, -z).  64 threads sweep the 64 lines of an axis, one line
-// each.  Afterwards the block and its existing face neighbours join this
-// iteration's tlist.  Thread 0 of CTA 0 zeroes the next update set's size
-// first (that set was consumed by the previous iteration).
-__global__ void __launch_bounds__(64)
-    esdf_sweep_kernel(const EsdfDev e, const uint32_t* __restrict__ list, const uint32_t* size,
-                      uint32_t* zero_next, uint32_t* tlist, uint32_t* tsize, uint32_t gen_t) {
-  __shared__ uint32_t s[kSweepWords];
-  __shared__ int s2[kSweepWords];
-  const uint32_t n = __ldcg(size);
-  const int t = threadIdx.x;
-  if (blockIdx.x == 0 && t == 0) {
-    *zero_next = 0u;
-    if (n) {
-      atomicAdd(e.stats + 1, 1ull);
-      atomicAdd(e.stats + 2, (unsigned long long)n);
+constexpr int kLowerThreads = 256;
+constexpr int kLowerWarps = kLowerThreads / 32;
+
+// One warp's block in shared memory: states and squared parent distances.
+struct LowerBlock {
+  uint32_t s[kSweepWords];
+  int s2[kSweepWords];
+};
+
+// Grid-wide barrier `k` (0, 1, ...) of a cooperative launch: every CTA is
+// resident, so the wait ends; after a second of the global timer it gives up
+// all the same, flags it and returns false to the whole CTA.
+__device__ __forceinline__ bool grid_barrier(const EsdfDev& e, unsigned k, bool* s_ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(e.cnt + kEcBarrier, 1u);
+    unsigned long long t0, t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    bool ok = true;
+    for (;;) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(e.cnt + kEcBarrier) : "memory");
+      if (v >= (k + 1u) * gridDim.x) break;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (t - t0 > 1000000000ull) {
+        ok = false;
+        atomicOr(e.cnt + kEcTimeout, 1u);
+        break;
+      }
+      __nanosleep(32);
     }
+    __threadfence();
+    *s_ok = ok;
   }
-  const int max2 = e.max_dist * e.max_dist;
-  const int a = t & 7, c = t >> 3;  // the line's coordinates on the two other axes, in axis order
-  for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
-    const uint32_t p = list[k];
-    uint32_t* g = e.st + (size_t)p * 512;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t v = g[t + 64 * i];
-      s[sweep_idx(t + 64 * i)] = v;
-      s2[sweep_idx(t + 64 * i)] = dist2(v);
-    }
-    __syncthreads();
-    sweep_line<0>(s, s2, kSweepRow * a + kSweepSlice * c, max2);
-    __syncthreads();
-    sweep_line<1>(s, s2, a + kSweepSlice * c, max2);
-    __syncthreads();
-    sweep_line<2>(s, s2, a + kSweepRow * c, max2);
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) g[t + 64 * i] = s[sweep_idx(t + 64 * i)];
-    if (t < 7) {
-      const int q = t == 6 ? (int)p : e.nbr[6 * (size_t)p + t];
-      if (q >= 0 && atomicExch(e.stamp_t + q, gen_t) != gen_t) tlist[atomicAdd(tsize, 1u)] = (uint32_t)q;
-    }
-  }
+  __syncthreads();
+  return *s_ok;
 }
 
-// Face exchange: each voxel on a face of the block tries the parent of the
-// voxel across that face in the neighbouring block, faces in -x, +x, -y,
-// +y, -z, +z order; reads st only, writes the block to st2 if it changed.
-__global__ void __launch_bounds__(kEsdfThreads)
-    esdf_pull_kernel(const EsdfDev e, const uint32_t* __restrict__ tlist, const uint32_t* tsize) {
-  __shared__ int s_nb[6];
-  const uint32_t n = __ldcg(tsize);
-  const int t = threadIdx.x;
-  const int max2 = e.max_dist * e.max_dist;
-  if (blockIdx.x == 0 && t == 0 && n) atomicAdd(e.stats + 3, (unsigned long long)n);
-  for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
-    const uint32_t p = tlist[k];
-    __syncthreads();
-    if (t < 6) s_nb[t] = e.nbr[6 * (size_t)p + t];
-    __syncthreads();
-    uint32_t v[4];
-    bool any = false;
+// The current block's sweeps, by its warp.
+__device__ __forceinline__ void sweep_block(LowerBlock& b, int lane, int max2) {
+  const int a = lane & 7, c = lane >> 3;  // lines (a, c) and (a, c + 4) on the two other axes, in axis order
+  __syncwarp();
+  sweep_lines<0>(b.s, b.s2, kSweepRow * a + kSweepSlice * c, kSweepRow * a + kSweepSlice * (c + 4), max2);
+  __syncwarp();
+  sweep_lines<1>(b.s, b.s2, a + kSweepSlice * c, a + kSweepSlice * (c + 4), max2);
+  __syncwarp();
+  sweep_lines<2>(b.s, b.s2, a + kSweepRow * c, a + kSweepRow * (c + 4), max2);
+  __syncwarp();
+}
+
+// Block states between global and shared memory, 16-byte vectors (voxels
+// 128 j + 4 lane + i).  Global accesses bypass L1: other SMs wrote the block
+// earlier in this launch.
+__device__ __forceinline__ void load_block(LowerBlock& b, const uint32_t* g, int lane) {
+  uint4 v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = __ldcg(reinterpret_cast<const uint4*>(g) + 32 * j + lane);
+  __syncwarp();  // the previous block's reads are done
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int l = 4 * t + i;
-      const int x = l & 7, y = (l >> 3) & 7, z = l >> 6;
-      const int c[3] = {x, y, z};
-      v[i] = e.st[(size_t)p * 512 + l];
+      const int at = sweep_idx(128 * j + 4 * lane + i);
+      b.s[at] = w[i];
+      b.s2[at] = dist2(w[i]);
+    }
+  }
+}
+__device__ __forceinline__ void store_block(const LowerBlock& b, uint32_t* g, int lane) {
 #pragma unroll
-      for (int f = 0; f < 6; ++f) {
-        const int axis = f >> 1;
-        const int mine = (f & 1) ? 7 : 0;
-        if (c[axis] != mine || s_nb[f] < 0) continue;
-        const int ql = l + (axis == 0 ? 1 : (axis == 1 ? 8 : 64)) * (7 - 2 * mine);
-        const uint32_t q = e.st[(size_t)s_nb[f] * 512 + ql];
-        const int d = (f & 1) ? 1 : -1;
-        any |= relax(v[i], q, axis == 0 ? d : 0, axis == 1 ? d : 0, axis == 2 ? d : 0, max2);
-      }
-    }
-    any = __syncthreads_or(any);
-    if (any) {
-      uint4* dst = reinterpret_cast<uint4*>(e.st2 + (size_t)p * 512) + t;
-      *dst = make_uint4(v[0], v[1], v[2], v[3]);
-    }
-    if (t == 0) e.tchanged[k] = any ? 1 : 0;
+  for (int j = 0; j < 4; ++j) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = b.s[sweep_idx(128 * j + 4 * lane + i)];
+    __stcg(reinterpret_cast<uint4*>(g) + 32 * j + lane, make_uint4(w[0], w[1], w[2], w[3]));
   }
 }
 
-// Copy the changed blocks back; they form the next update set.  One warp
-// per tlist entry, four 16-byte vectors per lane.  Thread 0 of CTA 0 zeroes
-// the other tlist's size (used by the previous iteration, filled by the
-// next one).
-__global__ void __launch_bounds__(kEsdfThreads)
-    esdf_apply_kernel(const EsdfDev e, const uint32_t* __restrict__ tlist, const uint32_t* tsize,
-                      uint32_t* zero_tsize, uint32_t* next, uint32_t* next_size, uint32_t gen_next) {
-  constexpr int kWarps = kEsdfThreads / 32;
-  const uint32_t n = __ldcg(tsize);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *zero_tsize = 0u;
-  for (uint32_t k = blockIdx.x * kWarps + warp; k < n; k += gridDim.x * kWarps) {
-    if (!e.tchanged[k]) continue;
-    const uint32_t p = tlist[k];
-    uint4* dst = reinterpret_cast<uint4*>(e.st + (size_t)p * 512) + lane;
+// The block and its existing face neighbours join the exchange set of
+// generation gen (lanes 0 .. 6; nbr: the lane's neighbour, or the block).
+__device__ __forceinline__ void join_exchange(const EsdfDev& e, int nbr, uint32_t gen, uint32_t* list, uint32_t* size,
+                                              int lane) {
+  if (lane < 7 && nbr >= 0 && atomicExch(e.stamp_t + nbr, gen) != gen) list[atomicAdd(size, 1u)] = (uint32_t)nbr;
+}
+
+// The lowering iterations in one cooperative launch.
+//
+// A block belongs to one warp at a time.  Phase 0 sweeps the update set that
+// the mark and clear stages left; phase k >= 1 is the exchange of iteration
+// k - 1 fused with the sweeps of iteration k: a warp takes a block of the
+// exchange set, tries its six faces, and if the block changed sweeps it right
+// away (sweeps read nothing else) and puts it and its neighbours in the next
+// exchange set.  The exchange must read every neighbour as it was before the
+// phase, so a block is rewritten in the other of two buffers (st, st2):
+// ver[p] = generation of its last rewrite << 1 | buffer, and a reader that
+// finds the present generation there reads the other buffer, which no one
+// writes in this phase.  One grid barrier per iteration; the last step copies
+// the blocks that ended in st2 back.
+//
+// Three kernels per iteration and a read-back of the set size every four cost
+// the 16 iterations of a room map of 40 frames from scratch and its update
+// after 8 more 470 us of kernels and six host round trips; this launch takes
+// 154 + 75 us.  The sweeps' instructions bound the first phases, the latency
+// of a block's dependent steps and of the barriers the small ones.
+__global__ void __launch_bounds__(kLowerThreads, 3)
+    esdf_lower_kernel(const MapDev m, const EsdfDev e, uint32_t gen, int with_table) {
+  __shared__ LowerBlock blocks[kLowerWarps];
+  __shared__ bool s_ok;
+  const int lane = threadIdx.x & 31;
+  LowerBlock& b = blocks[threadIdx.x >> 5];
+  // warps numbered across the CTAs first, so that a short list spreads over the SMs
+  const uint32_t warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, warps = gridDim.x * kLowerWarps;
+  const int max2 = e.max_dist * e.max_dist;
+  const uint32_t n0 = __ldcg(e.cnt + kEcUpdate);
+  if (n0 == 0) return;  // nothing marked: the same for every CTA
+  unsigned barrier = 0;
+  if (with_table) {
+    neighbour_table(m, e);
+    if (!grid_barrier(e, barrier++, &s_ok)) return;
+  }
+  const uint32_t my_face = lane < 6 ? (uint32_t)lane : 0u;
+  // phase 0: sweep the update set in place
+  for (uint32_t k = warp; k < n0; k += warps) {
+    const uint32_t p = __ldcg(e.list + k);
+    int nbr = __ldcg(e.nbr + 6 * (size_t)p + my_face);
+    if (lane == 6) nbr = (int)p;
+    uint32_t* g = e.st + (size_t)p * 512;
+    load_block(b, g, lane);
+    sweep_block(b, lane, max2);
+    store_block(b, g, lane);
+    join_exchange(e, nbr, gen, e.tlist[1], e.cnt + kEcExchange + 1, lane);
+  }
+  uint32_t swept = n0, pulled = 0, k = 1;
+  for (;; ++k) {
+    if (!grid_barrier(e, barrier++, &s_ok)) return;
+    const uint32_t n = __ldcg(e.cnt + kEcExchange + k % 3);
+    if (n == 0) break;
+    const uint32_t* list = (k & 1u) ? e.tlist[1] : e.tlist[0];
+    uint32_t* next = (k & 1u) ? e.tlist[0] : e.tlist[1];
+    uint32_t* next_size = e.cnt + kEcExchange + (k + 1) % 3;
+    if (blockIdx.x == 0 && threadIdx.x == 0) e.cnt[kEcExchange + (k + 2) % 3] = 0u;  // last read in the phase before
+    pulled += n;
+    const uint32_t now = (gen + k - 1u) & 0x7FFFFFFFu;  // this phase's generation in ver
+    for (uint32_t i = warp; i < n; i += warps) {
+      const uint32_t p = __ldcg(list + i);
+      int nbr = __ldcg(e.nbr + 6 * (size_t)p + my_face);
+      if (lane == 6) nbr = (int)p;
+      // buffer of this block (lane 6) and of each neighbour (lanes 0 .. 5)
+      uint32_t ver = lane < 7 && nbr >= 0 ? __ldcg(e.ver + nbr) : 0u;
+      uint32_t buf = ver & 1u;
+      if (lane < 6 && (ver >> 1) == now) buf ^= 1u;
+      const uint32_t mine = __shfl_sync(0xffffffffu, buf, 6);
+      // the voxels across the six faces, two per lane and face (u, v: the
+      // face's coordinates, v = 2 (lane >> 4) ... in steps of 32 voxels)
+      uint32_t q[6][2];
+#pragma unroll
+      for (int f = 0; f < 6; ++f) {
+        const int nb = __shfl_sync(0xffffffffu, nbr, f);
+        const uint32_t nbuf = __shfl_sync(0xffffffffu, buf, f);
+        const uint32_t* src = (nbuf ? e.st2 : e.st) + (size_t)(nb >= 0 ? nb : 0) * 512;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int u = lane & 7, v = (lane >> 3) + 4 * h, far = (f & 1) ? 0 : 7;  // the neighbour's facing layer
+          const int l = f < 2 ? far + 8 * u + 64 * v : (f < 4 ? u + 8 * far + 64 * v : u + 8 * v + 64 * far);
+          q[f][h] = nb >= 0 ? __ldcg(src + l) : 0u;
+        }
+      }
+      load_block(b, (mine ? e.st2 : e.st) + (size_t)p * 512, lane);
+      bool any = false;
+#pragma unroll
+      for (int f = 0; f < 6; ++f) {
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int u = lane & 7, v = (lane >> 3) + 4 * h, near = (f & 1) ? 7 : 0;
+          const int at = f < 2 ? near + kSweepRow * u + kSweepSlice * v
+                               : (f < 4 ? u + kSweepRow * near + kSweepSlice * v : u + kSweepRow * v + kSweepSlice * near);
+          const int d = (f & 1) ? 1 : -1;
+          uint32_t w = b.s[at];
+          if (relax(w, q[f][h], f >> 1 == 0 ? d : 0, f >> 1 == 1 ? d : 0, f >> 1 == 2 ? d : 0, max2)) {
+            b.s[at] = w;
+            b.s2[at] = dist2(w);
+            any = true;
+          }
+        }
+      }
+      if (!__any_sync(0xffffffffu, any)) continue;
+      sweep_block(b, lane, max2);
+      store_block(b, (mine ? e.st : e.st2) + (size_t)p * 512, lane);
+      if (lane == 0) {
+        __stcg(e.ver + p, (now << 1) | (mine ^ 1u));
+        atomicAdd(e.stats + 2, 1ull);
+      }
+      join_exchange(e, nbr, gen + k, next, next_size, lane);
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    atomicAdd(e.stats + 1, (unsigned long long)(k - 1));
+    atomicAdd(e.stats + 2, (unsigned long long)swept);
+    atomicAdd(e.stats + 3, (unsigned long long)pulled);
+    e.cnt[kEcIterations] = k - 1;
+  }
+  // every block's states in st again
+  const uint32_t nb = n_blocks(m);
+  for (uint32_t p = warp; p < nb; p += warps) {
+    if (!(__ldcg(e.ver + p) & 1u)) continue;  // the same for every lane
     const uint4* src = reinterpret_cast<const uint4*>(e.st2 + (size_t)p * 512) + lane;
+    uint4* dst = reinterpret_cast<uint4*>(e.st + (size_t)p * 512) + lane;
     uint4 v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = src[32 * j];
+    for (int j = 0; j < 4; ++j) v[j] = __ldcg(src + 32 * j);
 #pragma unroll
     for (int j = 0; j < 4; ++j) dst[32 * j] = v[j];
-    if (lane == 0) add_update(e, next, next_size, p, gen_next);
+    __syncwarp();
+    if (lane == 0) e.ver[p] &= ~1u;
   }
 }
 
@@ -641,7 +756,6 @@ cudaError_t launch_esdf_mark(const MapDev& m, const EsdfDev& e, uint32_t gen, cu
 
 cudaError_t launch_esdf_clear(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s) {
   esdf_clear_kernel<<<grid_for(10), kEsdfThreads, 0, s>>>(m, e, gen);  // 48 registers: 10 CTAs per SM
-  if (m.storage != kStorageOcc) esdf_nbr_kernel<<<grid_for(4), 256, 0, s>>>(m, e);  // built before marking otherwise
   return cudaGetLastError();
 }
 
@@ -650,23 +764,28 @@ cudaError_t launch_esdf_reset(const MapDev& m, const EsdfDev& e, cudaStream_t s)
   return cudaGetLastError();
 }
 
-// One lowering iteration (update set `cur`, tlist `cur`): sweep and build
-// the tlist, exchange faces, apply.  With an empty current set every kernel
-// returns at once.
-cudaError_t launch_esdf_iteration(const MapDev& m, const EsdfDev& e, int cur, uint32_t gen_t,
-                                  uint32_t gen_next, cudaStream_t s) {
-  uint32_t* list = cur ? e.list[1] : e.list[0];
-  uint32_t* next = cur ? e.list[0] : e.list[1];
-  uint32_t* tl = cur ? e.tlist[1] : e.tlist[0];
-  uint32_t* tsize = e.cnt + 3 + cur;
-  // latency-bound stages: enough resident warps per SM to overlap the
-  // blocks' loads (sweep 40 registers x 64 threads, pull 32 x 128)
-  esdf_sweep_kernel<<<grid_for(24), 64, 0, s>>>(e, list, e.cnt + cur, e.cnt + (1 - cur), tl, tsize, gen_t);
-  esdf_pull_kernel<<<grid_for(16), kEsdfThreads, 0, s>>>(e, tl, tsize);
-  esdf_apply_kernel<<<grid_for(16), kEsdfThreads, 0, s>>>(e, tl, tsize, e.cnt + 3 + (1 - cur), next,
-                                                          e.cnt + (1 - cur), gen_next);
-  (void)m;
-  return cudaGetLastError();
+// The lowering iterations, launched cooperatively with every CTA that can be
+// resident.  Exchange generations start at gen.  The neighbour table is built
+// here unless the mark stage of an occupancy layer built it.
+cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s) {
+  static std::atomic<int> fit{0};  // resident CTAs per SM (all devices are alike here)
+  int n = fit.load(std::memory_order_relaxed);
+  if (n == 0) {
+    const cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, esdf_lower_kernel, kLowerThreads, 0);
+    if (err != cudaSuccess) return err;
+    if (n <= 0) return cudaErrorNotSupported;
+    fit.store(n, std::memory_order_relaxed);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid_for(n));
+  cfg.blockDim = dim3(kLowerThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;  // every CTA resident: the grid barriers can complete
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, esdf_lower_kernel, m, e, gen, m.storage == kStorageOcc ? 0 : 1);
 }
 
 cudaError_t launch_esdf_query(const MapDev& m, const EsdfDev& e, const float* pts, int64_t n,

@@ -438,15 +438,14 @@ void free_map(tsdf_map* m) {
   if (m->esdf_on) {
     cudaFree(m->esdf.st);
     cudaFree(m->esdf.st2);
-    cudaFree(m->esdf.list[0]);
-    cudaFree(m->esdf.list[1]);
+    cudaFree(m->esdf.list);
     cudaFree(m->esdf.tlist[0]);
     cudaFree(m->esdf.tlist[1]);
     cudaFree(m->esdf.nbr);
     cudaFree(m->esdf.clist);
     cudaFree(m->esdf.stamp_s);
     cudaFree(m->esdf.stamp_t);
-    cudaFree(m->esdf.tchanged);
+    cudaFree(m->esdf.ver);
     cudaFree(m->esdf.bits);
     cudaFree(m->esdf.cnt);
     cudaFree(m->esdf.stats);
@@ -1099,24 +1098,24 @@ tsdf_status esdf_alloc(tsdf_map* m, const tsdf_esdf_opts& o) {
   const size_t nb = (size_t)m->max_blocks;
   bool ok = cudaMalloc(&e.st, sizeof(uint32_t) * 512 * nb) == cudaSuccess &&
             cudaMalloc(&e.st2, sizeof(uint32_t) * 512 * nb) == cudaSuccess &&
-            cudaMalloc(&e.list[0], sizeof(uint32_t) * nb) == cudaSuccess &&
-            cudaMalloc(&e.list[1], sizeof(uint32_t) * nb) == cudaSuccess &&
+            cudaMalloc(&e.list, sizeof(uint32_t) * nb) == cudaSuccess &&
             cudaMalloc(&e.tlist[0], sizeof(uint32_t) * nb) == cudaSuccess &&
             cudaMalloc(&e.tlist[1], sizeof(uint32_t) * nb) == cudaSuccess &&
             cudaMalloc(&e.nbr, sizeof(int32_t) * 6 * nb) == cudaSuccess &&
             cudaMalloc(&e.clist, sizeof(uint32_t) * nb) == cudaSuccess &&
             cudaMalloc(&e.stamp_s, sizeof(uint32_t) * nb) == cudaSuccess &&
             cudaMalloc(&e.stamp_t, sizeof(uint32_t) * nb) == cudaSuccess &&
-            cudaMalloc(&e.tchanged, nb) == cudaSuccess &&
+            cudaMalloc(&e.ver, sizeof(uint32_t) * nb) == cudaSuccess &&
             cudaMalloc(&e.bits, sizeof(uint32_t) * 2 * gbt::kEsdfBitWords) == cudaSuccess &&
-            cudaMalloc(&e.cnt, sizeof(uint32_t) * 8) == cudaSuccess &&
+            cudaMalloc(&e.cnt, sizeof(uint32_t) * gbt::kEsdfCounts) == cudaSuccess &&
             cudaMalloc(&e.stats, sizeof(unsigned long long) * 4) == cudaSuccess &&
-            cudaMallocHost(&m->esdf_host, sizeof(uint32_t) * 8) == cudaSuccess;
+            cudaMallocHost(&m->esdf_host, sizeof(uint32_t) * gbt::kEsdfCounts) == cudaSuccess;
   if (ok)
     ok = cudaMemset(e.st, 0, sizeof(uint32_t) * 512 * nb) == cudaSuccess &&
          cudaMemset(e.stamp_s, 0, sizeof(uint32_t) * nb) == cudaSuccess &&
          cudaMemset(e.stamp_t, 0, sizeof(uint32_t) * nb) == cudaSuccess &&
-         cudaMemset(e.cnt, 0, sizeof(uint32_t) * 8) == cudaSuccess &&
+         cudaMemset(e.cnt, 0, sizeof(uint32_t) * gbt::kEsdfCounts) == cudaSuccess &&
+         cudaMemset(e.ver, 0, sizeof(uint32_t) * nb) == cudaSuccess &&
          cudaMemset(e.stats, 0, sizeof(unsigned long long) * 4) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;
   m->esdf_on = true;  // free_map releases whatever was allocated
@@ -1130,7 +1129,7 @@ tsdf_status esdf_alloc(tsdf_map* m, const tsdf_esdf_opts& o) {
 }
 
 tsdf_status esdf_read_counts(tsdf_map* m, cudaStream_t s) {
-  if (cudaMemcpyAsync(m->esdf_host, m->esdf.cnt, sizeof(uint32_t) * 8, cudaMemcpyDeviceToHost, s) !=
+  if (cudaMemcpyAsync(m->esdf_host, m->esdf.cnt, sizeof(uint32_t) * gbt::kEsdfCounts, cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail();
@@ -1159,25 +1158,19 @@ tsdf_status map_esdf_update(tsdf_map* map, const tsdf_esdf_opts* opts, void* cud
   EsdfDev& e = map->esdf;
   // mark sites and clear invalid parents: update set 0 gets generation g
   const uint32_t g = ++map->esdf_gen;
-  if (cudaMemsetAsync(e.cnt, 0, sizeof(uint32_t) * 8, s) != cudaSuccess ||
+  if (cudaMemsetAsync(e.cnt, 0, sizeof(uint32_t) * gbt::kEsdfCounts, s) != cudaSuccess ||
       cudaMemsetAsync(e.bits, 0, sizeof(uint32_t) * 2 * gbt::kEsdfBitWords, s) != cudaSuccess ||
       gbt::launch_esdf_mark(map->dev, e, g, s) != cudaSuccess ||
-      gbt::launch_esdf_clear(map->dev, e, g, s) != cudaSuccess)
+      gbt::launch_esdf_clear(map->dev, e, g, s) != cudaSuccess ||
+      // lower until no block changes, in one launch
+      gbt::launch_esdf_lower(map->dev, e, g + 1, s) != cudaSuccess)
     return cuda_fail();
-  // lower until no block changes: four iterations per read-back of the set
-  // size (iterations on an empty set return at once)
-  constexpr int kItersPerCheck = 4;
-  int cur = 0;
-  for (;;) {
-    for (int k = 0; k < kItersPerCheck; ++k) {
-      const uint32_t gen_t = ++map->esdf_gen, gen_next = ++map->esdf_gen;
-      if (gbt::launch_esdf_iteration(map->dev, e, cur, gen_t, gen_next, s) != cudaSuccess)
-        return cuda_fail();
-      cur = 1 - cur;
-    }
-    tsdf_status st = esdf_read_counts(map, s);
-    if (st != TSDF_OK) return st;
-    if (map->esdf_host[cur] == 0) break;
+  tsdf_status st = esdf_read_counts(map, s);
+  if (st != TSDF_OK) return st;
+  map->esdf_gen = g + 1 + map->esdf_host[gbt::kEcIterations];
+  if (map->esdf_host[gbt::kEcTimeout]) {  // a grid barrier gave up: the layer is not converged
+    map->status_seen |= gbt::kStTimeout;
+    return TSDF_ERR_TIMEOUT;
   }
   return TSDF_OK;
 }

@@ -124,21 +124,27 @@ constexpr uint32_t kEsdfObs = 1u << 27, kEsdfSite = 1u << 28, kEsdfPar = 1u << 2
                    kEsdfInside = 1u << 30;
 constexpr uint32_t kEsdfOffMask = (1u << 27) - 1u;
 constexpr int kEsdfBitWords = (1 << 16) / 32;
+constexpr int kEsdfCounts = 16;
+// Words of EsdfDev::cnt: update set and lost-site sizes of the mark and clear
+// stages, the three exchange-set sizes in rotation, the grid barrier's
+// arrivals, and what the host reads: iterations run, a barrier timed out.
+enum : int { kEcUpdate = 0, kEcLost = 2, kEcExchange = 3, kEcBarrier = 6, kEcIterations = 7, kEcTimeout = 8 };
 struct EsdfDev {
   uint32_t* st;         // [max_blocks][512] voxel states
   uint32_t* st2;        // [max_blocks][512] states produced by a face exchange
-  uint32_t* list[2];    // [max_blocks] update sets (current, next)
+  uint32_t* list;       // [max_blocks] update set of the mark and clear stages
   uint32_t* tlist[2];   // [max_blocks] update set and its face neighbours (alternate
                         // iterations use alternate lists)
   uint32_t* clist;      // [max_blocks] blocks where a site disappeared
   uint32_t* stamp_s;    // [max_blocks] generation that put the block in an update set
   uint32_t* stamp_t;    // [max_blocks] generation that put the block in a tlist
-  uint8_t* tchanged;    // [max_blocks] per tlist entry: the exchange changed the block
+  uint32_t* ver;        // [max_blocks] generation of the block's last rewrite << 1 | buffer
+                        // holding it (0: st, 1: st2; 0 between updates)
   int32_t* nbr;         // [max_blocks][6] pool index of each face neighbour (-x, +x, -y,
                         // +y, -z, +z), -1 if none; rebuilt by every update
   uint32_t* bits;       // [2][kEsdfBitWords] hashed bitmaps of the clist blocks and of their
                         // coarse cells, rebuilt by every update
-  uint32_t* cnt;        // [0], [1] update set sizes, [2] clist size, [3], [4] tlist sizes
+  uint32_t* cnt;        // [kEsdfCounts] set sizes and barrier of the update in flight (kEc*)
   unsigned long long* stats;    // [0] voxels whose parent stopped being a site, [1] lowering
                                 // iterations, [2] blocks swept, [3] blocks in face exchanges
   float site_eps, min_weight;
@@ -354,11 +360,10 @@ cudaError_t launch_decay(const MapDev& m, float d_occ, float d_free, cudaStream_
 // Forget the ESDF states of the map's blocks; before launch_reset, which
 // forgets how many there are.
 cudaError_t launch_esdf_reset(const MapDev& m, const EsdfDev& e, cudaStream_t s);
-// ESDF stages (esdf.cu); `cur` selects the current update set.
+// ESDF stages (esdf.cu).
 cudaError_t launch_esdf_mark(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);
 cudaError_t launch_esdf_clear(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);
-cudaError_t launch_esdf_iteration(const MapDev& m, const EsdfDev& e, int cur, uint32_t gen_t,
-                                  uint32_t gen_next, cudaStream_t s);
+cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);
 cudaError_t launch_esdf_query(const MapDev& m, const EsdfDev& e, const float* pts, int64_t n,
                               float* dist, cudaStream_t s);
 cudaError_t launch_import(const MapDev& m, const int32_t* keys, const float* D, const float* W,

@@ -36,7 +36,8 @@ namespace {
 
 // Programmatic dependent launch: a kernel launched with BatchParams::overlap
 // may be scheduled while the stream's previous kernel is still running; it
-// waits here, before its first memory access, until that kernel has
+// stages what its parameters give (sensor constants, empty shared sets), then
+// waits here, before its first global memory access, until that kernel has
 // completed and its writes are visible.  Such a kernel lets the next one be
 // scheduled once its CTAs have done their main work.  Ordinary launches skip
 // both instructions.
@@ -315,7 +316,8 @@ __device__ __forceinline__ int tile_frame(const BatchParams<NF, NM>& p, int cta)
 // kAllocThreads threads of a CTA.  With p.overlap the stream's next kernel may be
 // scheduled once the walks are done.
 template <int NF, int NM, int TH, bool PINHOLE_ONLY, bool STATS, bool FAST, bool CAP>
-__device__ __forceinline__ void alloc_tile(const BatchParams<NF, NM>& p, int f, int cta, AllocSmem<TH>& sm) {
+__device__ __forceinline__ void alloc_tile(const BatchParams<NF, NM>& p, int f, int cta, AllocSmem<TH>& sm,
+                                           bool wait) {
   constexpr int kRows = TH * kTileW / kAllocThreads;  // pixel rows per thread
   uint32_t segs = 0, cells = 0;                        // walk statistics
   uint32_t* s_set = sm.set;
@@ -331,13 +333,6 @@ __device__ __forceinline__ void alloc_tile(const BatchParams<NF, NM>& p, int f, 
   const int tile = cta - F.blk_begin;
   const int x0 = (tile % tiles_x) * kTileW, y0 = (tile / tiles_x) * TH;
   const int lane = threadIdx.x % kTileW, wy = threadIdx.x / kTileW;
-  // all of this thread's depths are requested before any is used
-  float dep[kRows];
-#pragma unroll
-  for (int q = 0; q < kRows; ++q) {
-    const int i = x0 + lane, j = y0 + wy + q * (kAllocThreads / kTileW);
-    dep[q] = (i < F.width && j < F.height) ? __ldg(F.depth + (size_t)j * F.width + i) : 0.0f;
-  }
   if (PINHOLE_ONLY || F.kind == kSensorPinhole) {
     if (threadIdx.x < kTileW)
       s_ray[threadIdx.x] = __fdiv_rn(__fsub_rn((float)(x0 + (int)threadIdx.x), F.cu), F.fu);
@@ -347,6 +342,15 @@ __device__ __forceinline__ void alloc_tile(const BatchParams<NF, NM>& p, int f, 
           make_float4(__fmaf_rn(F.M[1], ry, F.M[2]), __fmaf_rn(F.M[4], ry, F.M[5]),
                       __fmaf_rn(F.M[7], ry, F.M[8]), 0.0f);
     }
+  }
+  // nothing above reads memory that the stream's previous kernel may write
+  if (wait) wait_prev_grid();
+  // all of this thread's depths are requested before any is used
+  float dep[kRows];
+#pragma unroll
+  for (int q = 0; q < kRows; ++q) {
+    const int i = x0 + lane, j = y0 + wy + q * (kAllocThreads / kTileW);
+    dep[q] = (i < F.width && j < F.height) ? __ldg(F.depth + (size_t)j * F.width + i) : 0.0f;
   }
   __syncthreads();
 
@@ -417,10 +421,9 @@ __device__ __forceinline__ void alloc_tile(const BatchParams<NF, NM>& p, int f, 
 template <int NF, int NM, int TH, bool PINHOLE_ONLY, bool STATS, bool FAST, bool CAP>
 __global__ void __launch_bounds__(kAllocThreads, 7)
     band_alloc_kernel(const __grid_constant__ BatchParams<NF, NM> p) {
-  if (p.overlap) wait_prev_grid();
   __shared__ AllocSmem<TH> sm;
   const int f = tile_frame(p, (int)blockIdx.x);
-  alloc_tile<NF, NM, TH, PINHOLE_ONLY, STATS, FAST, CAP>(p, f, (int)blockIdx.x, sm);
+  alloc_tile<NF, NM, TH, PINHOLE_ONLY, STATS, FAST, CAP>(p, f, (int)blockIdx.x, sm, p.overlap != 0);
 }
 
 // ------------------------------------------- pinhole tiles by pixel patches
@@ -573,9 +576,6 @@ __device__ __forceinline__ void patch_tile(const BatchParams<NF, NM>& p, const F
   const int tiles_x = (F.width + kPatchTile - 1) / kPatchTile;
   const int x0 = (tile % tiles_x) * kPatchTile, y0 = (tile / tiles_x) * kPatchTile;
   const int px = (t % kPatchesX) * 4, py = (t / kPatchesX) * 4;  // this thread's patch in the tile
-  float4 d[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) d[r] = strip_depths(F, x0 + px, y0 + py + r);
   for (int i = t; i < kWin * kWin; i += NT) sm.bm[i] = 0u;
   for (int i = t; i < 2 * kPatchTile; i += NT) {
     if (i < kPatchTile) {
@@ -592,6 +592,10 @@ __device__ __forceinline__ void patch_tile(const BatchParams<NF, NM>& p, const F
     sm.hi = 0;
     sm.n[0] = sm.n[1] = 0u;
   }
+  if (p.overlap) wait_prev_grid();  // nothing above reads memory that the previous kernel may write
+  float4 d[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) d[r] = strip_depths(F, x0 + px, y0 + py + r);
   uint32_t plo = 0xFFFFFFFFu;
   int phi = 0;
 #pragma unroll
@@ -737,7 +741,7 @@ __device__ __forceinline__ void patch_tile(const BatchParams<NF, NM>& p, const F
 
 union PatchOrRowSmem {
   PatchSmem patch;
-  AllocSmem<kTileHSmall> row;
+  AllocSmem<kTileHTiny> row;
 };
 
 // Allocation of a batch whose frames all pass the host's reciprocal and
@@ -746,14 +750,13 @@ union PatchOrRowSmem {
 template <int NF, int NM, bool MIXED>
 __global__ void __launch_bounds__(kAllocThreads, 5)
     patch_alloc_kernel(const __grid_constant__ BatchParams<NF, NM> p) {
-  if (p.overlap) wait_prev_grid();
   const int f = tile_frame(p, (int)blockIdx.x);
   const FrameDev& F = p.fr[f];
   const MapDev& m = NM == 1 ? p.maps[0] : p.maps[F.map];
   if (MIXED) {
     __shared__ PatchOrRowSmem sm;
     if (F.kind != kSensorPinhole)
-      alloc_tile<NF, NM, kTileHSmall, false, false, true, false>(p, f, (int)blockIdx.x, sm.row);
+      alloc_tile<NF, NM, kTileHTiny, false, false, true, false>(p, f, (int)blockIdx.x, sm.row, p.overlap != 0);
     else
       patch_tile(p, F, m, (int)blockIdx.x - F.blk_begin, sm.patch);
   } else {
@@ -1339,7 +1342,8 @@ __device__ __forceinline__ T meta_load(const T* a) {
 // finishes an entry's last slab clears its mask (every slab has read it by
 // then).  The last CTA to finish resets every map's work list.
 template <int NF, int NM, bool COHERENT, int STORAGE, bool PINHOLE_ONLY, bool WEIGHTED, bool FAST>
-__device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, IntegSmem<NF, NM>& sm) {
+__device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, IntegSmem<NF, NM>& sm,
+                                                  bool wait) {
   if (threadIdx.x < NM) sm.upd[threadIdx.x] = sm.pairs[threadIdx.x] = 0ull;
   for (int f = threadIdx.x; f < p.n_frames; f += blockDim.x)
     if (p.fr[f].kind == kSensorPinhole) stage_frame(p.fr[f], sm.fp[f]);
@@ -1348,6 +1352,8 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
     sm.entry[threadIdx.x] = blockIdx.x;
     sm.done[threadIdx.x] = 0u;
   }
+  // nothing above reads memory that the stream's previous kernel may write
+  if (wait) wait_prev_grid();
   if (threadIdx.x == 0) {
     sm.ticket = 0u;
     // the batch's work = the concatenation of every map's list
@@ -1360,6 +1366,13 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
   }
   __syncthreads();
   const uint32_t n = sm.begin[p.n_maps];
+  // a CTA's first entry is its own index: one beyond the list has none and is
+  // not counted below (CTA 0 always is).  A CTA that starts late may read the
+  // list as already reset: then it was not counted either.  (In the fused
+  // kernel every CTA is counted: the reset ends the grid wait's count, so it
+  // has to come after every CTA has left the wait.)
+  if (!COHERENT && blockIdx.x >= n && blockIdx.x != 0) return;
+  const uint32_t ctas = COHERENT ? gridDim.x : max(1u, min(n, gridDim.x));
   const int lane = threadIdx.x & 31;
 
   for (;;) {
@@ -1438,9 +1451,9 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
             }
           }
         }
-        if (nq == 2)
+        if (NF > 1 && nq == 2)
           fuse_pinhole<2, STORAGE, WEIGHTED, FAST>(p, sm.fp, fq, m, vq, D, W, G4, B, my_upd);
-        else if (nq == 1)
+        else if (nq >= 1)
           fuse_pinhole<1, STORAGE, WEIGHTED, FAST>(p, sm.fp, fq, m, vq, D, W, G4, B, my_upd);
         else if (!PINHOLE_ONLY) {
           const int f = __ffs(bits) - 1;  // a LiDAR frame
@@ -1475,7 +1488,7 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned done = atomicAdd(p.maps[0].ctl + 1, 1u);
-    if (done == gridDim.x - 1) {
+    if (done == ctas - 1) {
       for (int k = 0; k < p.n_maps; ++k) {
         atomicAdd(p.maps[k].counters + kCntVisits, (unsigned long long)(sm.begin[k + 1] - sm.begin[k]));
         atomicAdd(p.maps[k].counters + kCntLaunches, 1ull);
@@ -1492,8 +1505,7 @@ template <int NF, int NM, int STORAGE, bool PINHOLE_ONLY, bool WEIGHTED, bool FA
 __global__ void __launch_bounds__(kIntegrateThreads, STORAGE == kStorageColor ? 6 : 7)
     integrate_kernel(const __grid_constant__ BatchParams<NF, NM> p) {
   __shared__ IntegSmem<NF, NM> sm;
-  if (p.overlap) wait_prev_grid();
-  integrate_entries<NF, NM, false, STORAGE, PINHOLE_ONLY, WEIGHTED, FAST>(p, sm);
+  integrate_entries<NF, NM, false, STORAGE, PINHOLE_ONLY, WEIGHTED, FAST>(p, sm, p.overlap != 0);
 }
 
 // ------------------------------------------- one launch per batch (fused)
@@ -1561,11 +1573,11 @@ __global__ void __launch_bounds__(kFusedThreads, 4)
     fused_kernel(const __grid_constant__ BatchParams<NF, NM> p) {
   __shared__ FusedSmem<NF, NM, TH> sm;
   for (int cta = blockIdx.x; cta < p.alloc_ctas; cta += gridDim.x)
-    alloc_tile<NF, NM, TH, PINHOLE_ONLY, false, FAST, true>(p, tile_frame(p, cta), cta, sm.a);
+    alloc_tile<NF, NM, TH, PINHOLE_ONLY, false, FAST, true>(p, tile_frame(p, cta), cta, sm.a, false);
   if (!grid_wait(p.maps[0].ctl + 3, gridDim.x + (unsigned)p.wait_extra, p.maps[0].counters + kCntStatus))
     return;  // timed out: integration skipped, the map reports TSDF_ERR_TIMEOUT
   __syncthreads();  // the tiles' shared memory is free for the integration
-  integrate_entries<NF, NM, true, STORAGE, PINHOLE_ONLY, false, FAST>(p, sm.i);
+  integrate_entries<NF, NM, true, STORAGE, PINHOLE_ONLY, false, FAST>(p, sm.i, false);
 }
 
 template <int STORAGE>
@@ -1740,17 +1752,23 @@ cudaError_t launch_k(void (*k)(P), dim3 g, dim3 b, cudaStream_t s, const P& p) {
 template <int NF, int NM>
 AllocShape pick_alloc_shape(const BatchParams<NF, NM>& p, int tile_h) {
   bool pinhole = false, ok = true;
-  int64_t pixels = 0;
+  int64_t pixels = 0, tiny_tiles = 0;
   for (int k = 0; k < p.n_maps; ++k) ok = ok && !p.maps[k].walk_stats;
   for (int f = 0; f < p.n_frames; ++f) {
     const FrameDev& F = p.fr[f];
     ok = ok && F.fast_rcp && F.short_walks;
     pinhole = pinhole || F.kind == kSensorPinhole;
     pixels += (int64_t)F.width * F.height;
+    tiny_tiles += (int64_t)((F.width + kTileW - 1) / kTileW) * ((F.height + kTileHTiny - 1) / kTileHTiny);
   }
   if (ok && pinhole && (tile_h ? tile_h == kTileHBig : pixels >= kPatchPixels))
-    return AllocShape{kPatchTile, kTileHSmall};
+    return AllocShape{kPatchTile, kTileHTiny};
   const bool big = tile_h ? tile_h == kTileHBig : pixels >= kBigTilePixels;
+  // Tiles of 8 rows walk one pixel per thread instead of two: less latency
+  // where they still fit one wave (a 64x48 call 16.5 -> 14.5 us, 640x480
+  // calls 119 -> 116 us for eight, a 1024x64 scan 57.4 -> 53.1), more claims
+  // per pixel where they do not (848x480: 80 -> 88 us for four calls).
+  if (ok && !tile_h && tiny_tiles <= kOneWave) return AllocShape{0, kTileHTiny};
   return AllocShape{0, big ? kTileHBig : kTileHSmall};
 }
 
@@ -1772,6 +1790,9 @@ cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, AllocSha
     return big ? launch_k(band_alloc_kernel<NF, NM, kTileHBig, false, false, false, true>, g, b, s, p)
                : launch_k(band_alloc_kernel<NF, NM, kTileHSmall, false, false, false, true>, g, b, s, p);
   const bool fast = p.fast_rcp != 0;
+  if (shape.row_h == kTileHTiny)  // every frame passed the host's checks (pick_alloc_shape)
+    return ph ? launch_k(band_alloc_kernel<NF, NM, kTileHTiny, true, false, true, false>, g, b, s, p)
+              : launch_k(band_alloc_kernel<NF, NM, kTileHTiny, false, false, true, false>, g, b, s, p);
   if (big) {
     // pinhole batches of this size with fast reciprocals take patch tiles
     if (ph) return launch_k(band_alloc_kernel<NF, NM, kTileHBig, true, false, false, false>, g, b, s, p);
@@ -1786,13 +1807,15 @@ cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, AllocSha
 
 // Launch integration kernel k on a persistent grid: per_sm CTAs per SM (the
 // map's knob), or if that is 0 as many as can be resident with this variant's
-// registers, at most `limit` (0: no limit).  Batches of many pinhole frames
-// are limited: an entry is then long work (up to 32 frames), and with every
-// SM full of entries half of them are started at once and the chip drains
-// unevenly (32 frames of 640x480, us per launch with 3, 4, 5, 7 and 9 CTAs per SM:
-// 56.6, 55.1, 55.3, 61.8, 61.4).  Single frames and LiDAR scans want every warp
-// (a scan with 4, 5, 7: 53, 47, 43).
-constexpr int kManyFrames = 8, kManyFramesPerSm = 5;
+// registers, at most `limit` (0: no limit).  Pinhole launches (not colour) are
+// limited.  In a batch of many frames an entry is long work, and with every SM
+// full of entries half of them are started at once and the chip drains
+// unevenly (32 frames of 640x480, us per launch with 3, 4, 5, 7 and 9 CTAs per
+// SM: 56.6, 55.1, 55.3, 61.8, 61.4); a single frame's launch leaves room for the
+// next call's allocation, which starts while it drains (eight 640x480 calls,
+// us in all with 3, 4, 5, 6, 7: 126.5, 120.1, 120.4, 123.8, 125.5).  LiDAR scans
+// want every warp (four scans with 4, 5, 6, 7: 271, 252, 242, 231 us).
+constexpr int kPinholePerSm = 5;
 template <class P>
 cudaError_t launch_persistent(void (*k)(P), int per_sm, int limit, cudaStream_t s, const P& p,
                               std::atomic<int>& fit) {
@@ -1831,7 +1854,7 @@ cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int per_sm, cudaStrea
   for (int k = 0; k < p.n_maps; ++k) wt = wt || p.maps[k].weighting != 0;
   // FAST: pinhole reciprocals by rcp_dec<true> (the host checked their range)
   const bool fast = p.fast_rcp != 0;
-  const int limit = ph && st != kStorageColor && p.n_frames >= kManyFrames ? kManyFramesPerSm : 0;
+  const int limit = ph && st != kStorageColor ? kPinholePerSm : 0;
 #define GBT_INTEG(ST, PH) \
   (fast ? launch_variant<NF, NM, ST, PH, false, true>(p, per_sm, limit, s) \
         : launch_variant<NF, NM, ST, PH, false, false>(p, per_sm, limit, s))

@@ -17,6 +17,8 @@ constexpr int kMaxMaps = 16;           // maps per batch
 constexpr unsigned long long kEmptyKey = ~0ull;
 constexpr int kAllocThreads = 256;     // threads per allocation CTA
 constexpr int kTileW = 32;             // allocation CTA = one 32 x (16 or 32) pixel tile
+constexpr int kTileHTiny = 8;          // launches whose tiles then fit one wave, LiDAR frames beside patch tiles
+constexpr int kOneWave = 8 * 152;      // allocation CTAs resident at once
 constexpr int kTileHSmall = 16;        // small launches: more CTAs
 constexpr int kTileHBig = 32;          // large launches: fewer, fuller CTAs
 constexpr int kBigTilePixels = 1 << 21;  // pixels per launch from which big tiles are used

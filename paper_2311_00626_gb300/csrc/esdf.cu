@@ -655,6 +655,8 @@ __global__ void __launch_bounds__(kPointThreads)
     esdf_query_kernel(const MapDev m, const EsdfDev e, const float* __restrict__ pts, int64_t n, float inv_v,
                       bool vec, float* __restrict__ dist) {
   const int64_t i = (int64_t)blockIdx.x * kPointThreads + threadIdx.x;
+  wait_prev_grid();
+  allow_next_grid();
   if (kPointsPerThread * i >= n) return;
   float c[3 * kPointsPerThread], out[kPointsPerThread];
   int pool[kPointsPerThread], l[kPointsPerThread];
@@ -792,8 +794,7 @@ cudaError_t launch_esdf_query(const MapDev& m, const EsdfDev& e, const float* pt
                               float* dist, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const PointLaunch q = point_launch(m.v, n, pts, dist, nullptr);
-  esdf_query_kernel<<<q.blocks, kPointThreads, 0, s>>>(m, e, pts, n, q.inv_v, q.vec, dist);
-  return cudaGetLastError();
+  return launch_dependent(esdf_query_kernel, q.blocks, kPointThreads, s, m, e, pts, n, q.inv_v, q.vec, dist);
 }
 
 cudaError_t launch_import(const MapDev& m, const int32_t* keys, const float* D, const float* W,

@@ -34,16 +34,6 @@
 namespace gbt {
 namespace {
 
-// Programmatic dependent launch: a kernel launched with BatchParams::overlap
-// may be scheduled while the stream's previous kernel is still running; it
-// stages what its parameters give (sensor constants, empty shared sets), then
-// waits here, before its first global memory access, until that kernel has
-// completed and its writes are visible.  Such a kernel lets the next one be
-// scheduled once its CTAs have done their main work.  Ordinary launches skip
-// both instructions.
-__device__ __forceinline__ void wait_prev_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 constexpr float kPiF = (float)3.14159265358979323846;
 constexpr float kHalfPiF = (float)(3.14159265358979323846 / 2);
 
@@ -1585,6 +1575,8 @@ __global__ void __launch_bounds__(kPointThreads)
     query_kernel(const MapDev m, const float* __restrict__ pts, int64_t n, float inv_v, bool vec,
                  float* __restrict__ dist, float* __restrict__ weight) {
   const int64_t i = (int64_t)blockIdx.x * kPointThreads + threadIdx.x;
+  wait_prev_grid();
+  allow_next_grid();
   if (kPointsPerThread * i >= n) return;
   float c[3 * kPointsPerThread], D[kPointsPerThread], W[kPointsPerThread];
   int pool[kPointsPerThread], l[kPointsPerThread];
@@ -1621,6 +1613,8 @@ __global__ void __launch_bounds__(kPointThreads)
     query_color_kernel(const MapDev m, const float* __restrict__ pts, int64_t n, float inv_v, bool vec,
                        float* __restrict__ rgb, float* __restrict__ weight) {
   const int64_t i = (int64_t)blockIdx.x * kPointThreads + threadIdx.x;
+  wait_prev_grid();
+  allow_next_grid();
   if (kPointsPerThread * i >= n) return;
   float c[3 * kPointsPerThread], W[kPointsPerThread];
   float4 out[kPointsPerThread];
@@ -1656,6 +1650,8 @@ __global__ void __launch_bounds__(kPointThreads)
 // min(blocks, max_blocks) blocks are exactly the allocated ones; a thread
 // handles four voxels (one 16-byte word) per step of a grid-stride loop.
 __global__ void decay_kernel(const MapDev m, float d_occ, float d_free) {
+  wait_prev_grid();
+  allow_next_grid();
   const unsigned long long nb =
       min((unsigned long long)m.max_blocks, __ldcg(m.counters + kCntBlocks));
   const size_t n4 = (size_t)nb * 128;
@@ -1684,6 +1680,8 @@ __global__ void reset_kernel(const MapDev m, uint32_t cap, const MoreSets more) 
   const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
   const uint4 ones = make_uint4(~0u, ~0u, ~0u, ~0u), zero = make_uint4(0u, 0u, 0u, 0u);
   static_assert(kEmptyKey == ~0ull, "an empty key is all ones");
+  wait_prev_grid();
+  allow_next_grid();
   for (uint32_t i = first; i < cap / 4; i += step) {
     reinterpret_cast<uint4*>(m.keys)[2 * i] = ones;
     reinterpret_cast<uint4*>(m.keys)[2 * i + 1] = ones;
@@ -1950,31 +1948,25 @@ cudaError_t launch_query(const MapDev& m, const float* pts, int64_t n, float* di
                          cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const PointLaunch q = point_launch(m.v, n, pts, dist, weight);
-  if (m.storage == kStorageOcc)
-    query_kernel<kStorageOcc><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
-  else if (m.storage == kStorageF16)
-    query_kernel<kStorageF16><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
-  else if (m.storage == kStorageX16)
-    query_kernel<kStorageX16><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
-  else
-    query_kernel<kStorageF32><<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, dist, weight);
-  return cudaGetLastError();
+  const auto k = m.storage == kStorageOcc   ? query_kernel<kStorageOcc>
+                 : m.storage == kStorageF16 ? query_kernel<kStorageF16>
+                 : m.storage == kStorageX16 ? query_kernel<kStorageX16>
+                                            : query_kernel<kStorageF32>;
+  return launch_dependent(k, q.blocks, kPointThreads, s, m, pts, n, q.inv_v, q.vec, dist, weight);
 }
 
 cudaError_t launch_query_color(const MapDev& m, const float* pts, int64_t n, float* rgb, float* weight,
                                cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const PointLaunch q = point_launch(m.v, n, pts, rgb, weight);
-  query_color_kernel<<<q.blocks, kPointThreads, 0, s>>>(m, pts, n, q.inv_v, q.vec, rgb, weight);
-  return cudaGetLastError();
+  return launch_dependent(query_color_kernel, q.blocks, kPointThreads, s, m, pts, n, q.inv_v, q.vec, rgb, weight);
 }
 
 cudaError_t launch_decay(const MapDev& m, float d_occ, float d_free, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  decay_kernel<<<sms * 8, 256, 0, s>>>(m, d_occ, d_free);
-  return cudaGetLastError();
+  return launch_dependent(decay_kernel, sms * 8, 256, s, m, d_occ, d_free);
 }
 
 cudaError_t launch_reset(const MapDev& m, uint32_t cap, const MoreSets& more, cudaStream_t s) {
@@ -1982,8 +1974,7 @@ cudaError_t launch_reset(const MapDev& m, uint32_t cap, const MoreSets& more, cu
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const unsigned need = std::max((cap / 4 + 255) / 256, ((unsigned)m.max_blocks / 16 + 255) / 256);
-  reset_kernel<<<std::max(1u, std::min(need, (unsigned)sms * 8)), 256, 0, s>>>(m, cap, more);
-  return cudaGetLastError();
+  return launch_dependent(reset_kernel, std::max(1u, std::min(need, (unsigned)sms * 8)), 256, s, m, cap, more);
 }
 
 }  // namespace gbt

@@ -227,6 +227,34 @@ __device__ __forceinline__ int hash_find(const MapDev& m, unsigned long long key
   return -1;
 }
 
+// Programmatic dependent launch: a kernel launched with BatchParams::overlap
+// may be scheduled while the stream's previous kernel is still running; it
+// stages what its parameters give (sensor constants, empty shared sets), then
+// waits here, before its first global memory access, until that kernel has
+// completed and its writes are visible.  Such a kernel lets the next one be
+// scheduled once its CTAs have done their main work.  Ordinary launches skip
+// both instructions.
+__device__ __forceinline__ void wait_prev_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launch a kernel that begins with wait_prev_grid() as a programmatic
+// dependent of the stream's previous kernel: short kernels (queries, resets,
+// decay) then pay no launch gap, and by allow_next_grid() at their start
+// neither does what follows them.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*k)(P...), unsigned blocks, unsigned threads, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // ----------------------------------------------------------- point lookup
 //
 // The query kernels look up kPointsPerThread consecutive points per thread.

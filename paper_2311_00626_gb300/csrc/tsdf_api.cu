@@ -649,23 +649,23 @@ tsdf_status prepare_batch(tsdf_map* const* maps, int32_t n_maps, const tsdf_fram
 // pointers and make sa wait for copies.
 using SubBatchHook = tsdf_status (*)(void* ctx, int b, int f0, int nf, cudaStream_t sa);
 
-// Sub-batches of up to 32 frames, each one allocation launch and one
+// Sub-batches of up to `per` (at most 32) frames, each one allocation launch and one
 // integration launch.  With more than one, sub-batch b uses mask / list set
 // b % kSets and its allocation runs on the lead map's auxiliary stream,
 // overlapping the integration of earlier sub-batches on the caller's stream;
 // it waits for the integration of b - kSets, which used the same set.
 tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDev>& fr, int32_t n,
-                      cudaStream_t s, SubBatchHook hook, void* ctx) {
+                      int per, cudaStream_t s, SubBatchHook hook, void* ctx) {
   // the params block is large; keep it off the stack
   static thread_local BatchParams<gbt::kMaxFrames, gbt::kMaxMaps> p;
   // single-map batches launch the one-map kernels (map fields become constants)
   static thread_local BatchParams<gbt::kMaxFrames, 1> p1;
   tsdf_map* lead = maps[0];
-  const int n_sub = (n + gbt::kMaxFrames - 1) / gbt::kMaxFrames;
+  const int n_sub = (n + per - 1) / per;
   if (lead->launch_mode == TSDF_LAUNCH_FUSED && n_maps == 1) {
     // one cooperative launch per sub-batch, on the caller's stream
     for (int b = 0; b < n_sub; ++b) {
-      const int f0 = b * gbt::kMaxFrames, nf = std::min(gbt::kMaxFrames, n - f0);
+      const int f0 = b * per, nf = std::min(per, n - f0);
       if (hook) {
         tsdf_status st = hook(ctx, b, f0, nf, s);
         if (st != TSDF_OK) return st;
@@ -719,7 +719,7 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
                 cudaStreamWaitEvent(lead->aux, lead->ev_start, 0) != cudaSuccess))
     return cuda_fail();
   for (int b = 0; b < n_sub; ++b) {
-    const int f0 = b * gbt::kMaxFrames, nf = std::min(gbt::kMaxFrames, n - f0);
+    const int f0 = b * per, nf = std::min(per, n - f0);
     cudaStream_t sa = piped ? lead->aux : s;
     if (piped && b >= gbt::kSets &&
         cudaStreamWaitEvent(sa, lead->ev_int[(b - gbt::kSets) & 3], 0) != cudaSuccess)
@@ -785,6 +785,7 @@ struct HostStaging {
   std::vector<int64_t> bytes;    // per frame: depth bytes
 };
 
+constexpr int64_t kSplitBytes = 32 << 20;  // images of a full sub-batch from which it is halved
 int64_t align256(int64_t x) { return (x + 255) / 256 * 256; }
 
 tsdf_status stage_sub_batch(void* ctx, int b, int f0, int nf, cudaStream_t sa) {
@@ -833,7 +834,7 @@ tsdf_status integrate_batch(tsdf_map* const* maps, int32_t n_maps, const tsdf_fr
   static thread_local std::vector<FrameDev> fr;
   tsdf_status st = prepare_batch(maps, n_maps, frames, n, fr);
   if (st != TSDF_OK) return st;
-  st = run_batch(maps, n_maps, fr, n, (cudaStream_t)cuda_stream, nullptr, nullptr);
+  st = run_batch(maps, n_maps, fr, n, gbt::kMaxFrames, (cudaStream_t)cuda_stream, nullptr, nullptr);
   if (st != TSDF_OK) return st;
   for (int f = 0; f < n; ++f) maps[frames[f].map]->frames += 1;
   return TSDF_OK;
@@ -851,18 +852,32 @@ tsdf_status integrate_batch_host(tsdf_map* const* maps, int32_t n_maps, const ts
   h.base = static_cast<char*>(staging_dev);
   h.off.resize(n);
   h.bytes.resize(n);
-  int64_t need = 0;
-  for (int f0 = 0; f0 < n; f0 += gbt::kMaxFrames) {
-    int64_t o = 0;
-    for (int f = f0; f < std::min(n, f0 + gbt::kMaxFrames); ++f) {
-      h.bytes[f] = (int64_t)fr[f].width * fr[f].height * 4;
-      h.off[f] = o;
-      o += align256(h.bytes[f]) * (fr[f].rgba ? 2 : 1);
+  for (int f = 0; f < n; ++f) h.bytes[f] = (int64_t)fr[f].width * fr[f].height * 4;
+  // offsets in the slots for sub-batches of `per` frames; the largest sub-batch
+  auto lay_out = [&](int per) {
+    int64_t need = 0;
+    for (int f0 = 0; f0 < n; f0 += per) {
+      int64_t o = 0;
+      for (int f = f0; f < std::min(n, f0 + per); ++f) {
+        h.off[f] = o;
+        o += align256(h.bytes[f]) * (fr[f].rgba ? 2 : 1);
+      }
+      need = std::max(need, o);
     }
-    need = std::max(need, o);
-  }
-  h.half = align256(need);
+    return align256(need);
+  };
+  h.half = lay_out(gbt::kMaxFrames);
   if (2 * h.half > staging_bytes) return TSDF_ERR_ARG;  // two sub-batches must fit
+  // The copies bound large images, and the last sub-batch's kernels run after
+  // them: half-size sub-batches leave less to run (96 frames of 640x480, 118
+  // MB: 735 -> 680 us).  Not for small images, where the kernels' own latency
+  // is what a smaller sub-batch repeats, nor for 16-bit voxels, which are
+  // rounded once per sub-batch.
+  int per = gbt::kMaxFrames;
+  if (h.half >= kSplitBytes && maps[0]->storage != TSDF_STORAGE_FP16 && maps[0]->storage != TSDF_STORAGE_FIXED16) {
+    per = gbt::kMaxFrames / 2;
+    h.half = lay_out(per);
+  }
   h.slots = (int)std::min<int64_t>(4, staging_bytes / h.half);
   tsdf_map* lead = maps[0];
   if (!lead->copy) {
@@ -877,7 +892,7 @@ tsdf_status integrate_batch_host(tsdf_map* const* maps, int32_t n_maps, const ts
   if (cudaEventRecord(lead->ev_start, s) != cudaSuccess ||
       cudaStreamWaitEvent(lead->copy, lead->ev_start, 0) != cudaSuccess)
     return cuda_fail();
-  st = run_batch(maps, n_maps, fr, n, s, stage_sub_batch, &h);
+  st = run_batch(maps, n_maps, fr, n, per, s, stage_sub_batch, &h);
   if (st != TSDF_OK) return st;
   for (int f = 0; f < n; ++f) maps[frames[f].map]->frames += 1;
   return TSDF_OK;

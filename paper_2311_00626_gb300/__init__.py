@@ -102,6 +102,8 @@ _lib = None
 def lib():
     """Load (building first if stale) the CUDA library; raises if impossible."""
     global _lib
+    if _lib is not None:  # set once, complete: no lock on every call
+        return _lib
     with _lock:
         if _lib is None:
             path = build_library()
@@ -160,11 +162,18 @@ def _pose(T) -> ctypes.Array:
     return (ctypes.c_double * 16)(*a.tolist())
 
 
+_PoseBuffer = ctypes.c_double * 16
+_F64 = np.dtype(np.float64)
+
+
 def _pose_arg(T):
     """A pose as a call argument: the array's own memory when it already is
     16 contiguous doubles (the caller holds it for the call), else a copy."""
-    if type(T) is np.ndarray and T.dtype == np.float64 and T.size == 16 and T.flags.c_contiguous:
-        return T.ctypes.data
+    if type(T) is np.ndarray and T.dtype == _F64 and T.size == 16 and T.flags.c_contiguous:
+        try:
+            return _PoseBuffer.from_buffer(T)  # half the time of T.ctypes.data
+        except (TypeError, ValueError):  # a read-only array
+            return T.ctypes.data
     return _pose(T)
 
 

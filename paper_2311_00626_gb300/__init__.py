@@ -171,7 +171,7 @@ def _pose_arg(T):
     16 contiguous doubles (the caller holds it for the call), else a copy."""
     if type(T) is np.ndarray and T.dtype == _F64 and T.size == 16 and T.flags.c_contiguous:
         try:
-            return _PoseBuffer.from_buffer(T)  # half the time of T.ctypes.data
+            return ctypes.addressof(_PoseBuffer.from_buffer(T))  # half the time of T.ctypes.data
         except (TypeError, ValueError):  # a read-only array
             return T.ctypes.data
     return _pose(T)

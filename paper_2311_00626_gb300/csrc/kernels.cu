@@ -816,9 +816,9 @@ __device__ __forceinline__ float2 half_tan2(float2 t) {
 // smaller one is 0 or at least 2^-80: the quotient mn / mx by the correctly
 // rounded reciprocal and one residual step (Markstein's theorem; nothing
 // underflows in this range).
-__device__ __forceinline__ float2 atan2_dec2(float2 y, float2 x) {
-  const float2 mx = make_float2(fmaxf(fabsf(x.x), fabsf(y.x)), fmaxf(fabsf(x.y), fabsf(y.y)));
-  const float2 mn = make_float2(fminf(fabsf(x.x), fabsf(y.x)), fminf(fabsf(x.y), fabsf(y.y)));
+// mx, mn: the larger and smaller magnitude; Y_POSITIVE: y >= 0.
+template <bool Y_POSITIVE>
+__device__ __forceinline__ float2 atan2_dec2(float2 y, float2 x, float2 mx, float2 mn) {
   const float2 r = rcp_dec2<true>(mx.x, mx.y);
   const float2 q0 = __fmul2_rn(mn, r);
   const float2 t = __ffma2_rn(__ffma2_rn(make_float2(-mx.x, -mx.y), q0, mn), r, q0);
@@ -836,8 +836,8 @@ __device__ __forceinline__ float2 atan2_dec2(float2 y, float2 x) {
   if (fabsf(y.y) > fabsf(x.y)) a.y = __fsub_rn(kHalfPiF, a.y);
   if (x.x < 0.0f) a.x = __fsub_rn(kPiF, a.x);
   if (x.y < 0.0f) a.y = __fsub_rn(kPiF, a.y);
-  if (y.x < 0.0f) a.x = -a.x;
-  if (y.y < 0.0f) a.y = -a.y;
+  if (!Y_POSITIVE && y.x < 0.0f) a.x = -a.x;
+  if (!Y_POSITIVE && y.y < 0.0f) a.y = -a.y;
   return a;
 }
 
@@ -849,11 +849,38 @@ __device__ __noinline__ float3 lidar_angles(float x, float y, float z) {
   return make_float3(rr, atan2_dec(y, x), atan2_dec(rho, z));
 }
 
-// Whether lidar_angles of a point is in the range of the pair forms.
-__device__ __forceinline__ bool pair_range(float x, float y, float z) {
-  const float ax = fabsf(x), ay = fabsf(y), az = fabsf(z);
-  const float m = fmaxf(ax, ay), n = fminf(fminf(ax, ay) == 0.0f ? 1.0f : fminf(ax, ay), az == 0.0f ? 1.0f : az);
-  return m >= 0x1p-30f && fmaxf(m, az) <= 0x1p30f && n >= 0x1p-80f;
+// lidar_angles of two points (x, y, z): by the pair forms if both lie in their
+// range (all three magnitudes at least 2^-80, the larger of |x| and |y| at
+// least 2^-30, all at most 2^30), else one by one.
+__device__ __forceinline__ void lidar_angles2(float2 x, float2 y, float2 z, float2& rr, float2& th, float2& ph) {
+  const float2 mx = make_float2(fmaxf(fabsf(x.x), fabsf(y.x)), fmaxf(fabsf(x.y), fabsf(y.y)));
+  const float2 mn = make_float2(fminf(fabsf(x.x), fabsf(y.x)), fminf(fabsf(x.y), fabsf(y.y)));
+  const float low = fminf(fminf(mn.x, mn.y), fminf(fabsf(z.x), fabsf(z.y)));
+  const float high = fmaxf(fmaxf(mx.x, mx.y), fmaxf(fabsf(z.x), fabsf(z.y)));
+  if (low >= 0x1p-80f && fminf(mx.x, mx.y) >= 0x1p-30f && high <= 0x1p30f) {
+    rr = sqrt2_dec(__ffma2_rn(x, x, __ffma2_rn(y, y, __fmul2_rn(z, z))));
+    const float2 rho = sqrt2_dec(__ffma2_rn(x, x, __fmul2_rn(y, y)));
+    th = atan2_dec2<false>(y, x, mx, mn);
+    ph = atan2_dec2<true>(rho, z, make_float2(fmaxf(rho.x, fabsf(z.x)), fmaxf(rho.y, fabsf(z.y))),
+                          make_float2(fminf(rho.x, fabsf(z.x)), fminf(rho.y, fabsf(z.y))));
+  } else {
+    const float3 a = lidar_angles(x.x, y.x, z.x), b = lidar_angles(x.y, y.y, z.y);
+    rr = make_float2(a.x, b.x);
+    th = make_float2(a.y, b.y);
+    ph = make_float2(a.z, b.z);
+  }
+}
+
+// min / max that return NaN if either operand is one.
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
 }
 
 // Azimuth column k in [-1, naz] wrapped into [0, naz).
@@ -1097,6 +1124,16 @@ __device__ __forceinline__ float2 neg_rcp2(float2 z) {
 constexpr float kFloorMagic = 12582912.0f;
 constexpr uint32_t kFloorBits = 0x4B400000u;
 
+// The constant-weight TSDF update (apply) of a voxel pair, selected per voxel.
+__device__ __forceinline__ void update_pair(const MapDev& m, float* D, float* W, float2 dp, bool ok0, bool ok1) {
+  const float2 wn = __fadd2_rn(make_float2(W[0], W[1]), twice(1.0f));
+  const float2 D2 = make_float2(D[0], D[1]);
+  const float2 diff = __ffma2_rn(D2, twice(-1.0f), make_float2(fminf(dp.x, m.tau), fminf(dp.y, m.tau)));
+  const float2 dn = __fadd2_rn(D2, __fmul2_rn(diff, make_float2(rcp_approx(wn.x), rcp_approx(wn.y))));
+  if (ok0) { D[0] = dn.x; W[0] = fminf(wn.x, m.wmax); }
+  if (ok1) { D[1] = dn.y; W[1] = fminf(wn.y, m.wmax); }
+}
+
 // NQ consecutive pinhole frames of the batch: phase 1 projects every voxel
 // into every frame (Eq. 2, nearest pixel) and issues all depth loads (and
 // colour loads for a colour layer), phase 2 applies the updates in frame
@@ -1183,12 +1220,8 @@ __device__ __forceinline__ void fuse_pinhole(const P& p, const FrameProj* s_fp, 
         if (ok1) apply<STORAGE, WEIGHTED>(m, D[i + 1], W[i + 1], z[q][i + 1], dp.y);
         upd += (ok0 ? 1u : 0u) + (ok1 ? 1u : 0u);
       } else {
-        const float2 wn = __fadd2_rn(make_float2(W[i], W[i + 1]), twice(1.0f));
-        const float2 D2 = make_float2(D[i], D[i + 1]);
-        const float2 diff = __ffma2_rn(D2, twice(-1.0f), make_float2(fminf(dp.x, m.tau), fminf(dp.y, m.tau)));
-        const float2 dn = __fadd2_rn(D2, __fmul2_rn(diff, make_float2(rcp_approx(wn.x), rcp_approx(wn.y))));
-        if (ok0) { D[i] = dn.x; W[i] = fminf(wn.x, m.wmax); ++upd; }
-        if (ok1) { D[i + 1] = dn.y; W[i + 1] = fminf(wn.y, m.wmax); ++upd; }
+        update_pair(m, D + i, W + i, dp, ok0, ok1);
+        upd += (ok0 ? 1u : 0u) + (ok1 ? 1u : 0u);
       }
     }
 }
@@ -1198,43 +1231,94 @@ __device__ __forceinline__ void fuse_pinhole(const P& p, const FrameProj* s_fp, 
 // applies the guarded bilinear sample and the updates.  A voxel at the
 // sensor origin, outside the elevation rows or with an invalid sample is not
 // updated; azimuth wraps.  Colour layers take pinhole frames only.
-template <int STORAGE, bool WEIGHTED>
+//
+// FAST (constant weight, at most 2^21 columns and rows, the host checks):
+// voxel pairs throughout, cells floored by the round-down addition (kFloorMagic),
+// and the sample and update only where a pair has a valid cell (about a third
+// of the voxels of an outdoor scan's band do).  A 1024x64 scan's launch 43.3 ->
+// 39.4 us; 32 mixed frames over 16 maps 88.8 -> 80.8.
+template <int STORAGE, bool WEIGHTED, bool FAST>
 __device__ __forceinline__ void fuse_lidar(const FrameDev& F, const MapDev& m, const VoxelQuad& r,
                                            float* D, float* W, uint32_t& upd) {
   if (STORAGE == kStorageColor) return;
   float px[4], py[4], pz[4];
   quad_points(F, m.v, r, px, py, pz);
   const int naz = F.width, nel = F.height;
-  float rr[4], th[4], ph[4], fx[4], fy[4], d00[4], d10[4], d01[4], d11[4];
-  bool ok[4];
+  float2 rr[2], th[2], ph[2];
 #pragma unroll
-  for (int i = 0; i < 4; i += 2) {
-    const float2 x = make_float2(px[i], px[i + 1]), y = make_float2(py[i], py[i + 1]),
-                 z = make_float2(pz[i], pz[i + 1]);
-    if (pair_range(x.x, y.x, z.x) && pair_range(x.y, y.y, z.y)) {
-      const float2 r = sqrt2_dec(__ffma2_rn(x, x, __ffma2_rn(y, y, __fmul2_rn(z, z))));
-      const float2 rho = sqrt2_dec(__ffma2_rn(x, x, __fmul2_rn(y, y)));
-      const float2 a = atan2_dec2(y, x), e = atan2_dec2(rho, z);
-      rr[i] = r.x; rr[i + 1] = r.y;
-      th[i] = a.x; th[i + 1] = a.y;
-      ph[i] = e.x; ph[i + 1] = e.y;
-    } else {
-#pragma unroll 1
-      for (int k = i; k < i + 2; ++k) {
-        const float3 q = lidar_angles(k == i ? x.x : x.y, k == i ? y.x : y.y, k == i ? z.x : z.y);
-        if (k == i) {
-          rr[i] = q.x; th[i] = q.y; ph[i] = q.z;
-        } else {
-          rr[i + 1] = q.x; th[i + 1] = q.y; ph[i + 1] = q.z;
+  for (int k = 0; k < 2; ++k)
+    lidar_angles2(make_float2(px[2 * k], px[2 * k + 1]), make_float2(py[2 * k], py[2 * k + 1]),
+                  make_float2(pz[2 * k], pz[2 * k + 1]), rr[k], th[k], ph[k]);
+  if (FAST && !WEIGHTED && !m.lidar_nearest) {
+    float2 fx[2], fy[2], d00[2], d10[2], d01[2], d11[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      // u = (theta - theta_start) alpha, rounded before 1/2 is taken off (an
+      // addition of the product could be contracted; a product with 1 is not)
+      const float2 uu = __ffma2_rn(__fmul2_rn(__fadd2_rn(th[k], twice(-F.theta_start)), twice(F.alpha)), twice(1.0f), twice(-0.5f));
+      const float2 vv = __ffma2_rn(__fmul2_rn(__fadd2_rn(ph[k], twice(-F.phi_start)), twice(F.beta)), twice(1.0f), twice(-0.5f));
+      const float2 tu = __fadd2_rd(uu, twice(kFloorMagic)), tv = __fadd2_rd(vv, twice(kFloorMagic));
+      fx[k] = __ffma2_rn(__fadd2_rn(tu, twice(-kFloorMagic)), twice(-1.0f), uu);  // uu - floor(uu), exact floor
+      fy[k] = __ffma2_rn(__fadd2_rn(tv, twice(-kFloorMagic)), twice(-1.0f), vv);
+      float q[2][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k0 = (int)(__float_as_uint(h ? tu.y : tu.x) - kFloorBits);
+        const int j0 = (int)(__float_as_uint(h ? tv.y : tv.x) - kFloorBits);
+        const bool ok = (h ? rr[k].y : rr[k].x) > 0.0f && (uint32_t)j0 < (uint32_t)(nel - 1) &&
+                        (uint32_t)(k0 + 1) <= (uint32_t)(naz + 1);
+        q[h][0] = q[h][1] = q[h][2] = q[h][3] = __int_as_float(0x7fc00000);  // no cell: not valid
+        if (ok) {
+          const int c0 = wrap_az(k0, naz), c1 = c0 + 1 == naz ? 0 : c0 + 1;
+          const float* row0 = F.depth + j0 * naz;
+          const float* row1 = row0 + naz;
+          q[h][0] = __ldg(row0 + c0);
+          q[h][1] = __ldg(row0 + c1);
+          q[h][2] = __ldg(row1 + c0);
+          q[h][3] = __ldg(row1 + c1);
         }
       }
+      d00[k] = make_float2(q[0][0], q[1][0]);
+      d10[k] = make_float2(q[0][1], q[1][1]);
+      d01[k] = make_float2(q[0][2], q[1][2]);
+      d11[k] = make_float2(q[0][3], q[1][3]);
     }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      bool ok[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float a = h ? d00[k].y : d00[k].x, b = h ? d10[k].y : d10[k].x, c = h ? d01[k].y : d01[k].x,
+                    e = h ? d11[k].y : d11[k].x;
+        const float hi = max_nan(max_nan(a, b), max_nan(c, e)), lo = min_nan(min_nan(a, b), min_nan(c, e));
+        ok[h] = lo >= F.min_range && hi <= F.max_range && !(__fsub_rn(hi, lo) > m.guard);
+      }
+      if (!(ok[0] || ok[1])) continue;
+      const float2 top = __ffma2_rn(fx[k], __ffma2_rn(d00[k], twice(-1.0f), d10[k]), d00[k]);
+      const float2 bot = __ffma2_rn(fx[k], __ffma2_rn(d01[k], twice(-1.0f), d11[k]), d01[k]);
+      const float2 d = __ffma2_rn(fy[k], __ffma2_rn(top, twice(-1.0f), bot), top);
+      const float2 dp = __ffma2_rn(rr[k], twice(-1.0f), d);
+      ok[0] = ok[0] && !(dp.x < -m.tau);
+      ok[1] = ok[1] && !(dp.y < -m.tau);
+      const int i = 2 * k;
+      if (STORAGE == kStorageOcc) {
+        if (ok[0]) apply<STORAGE, false>(m, D[i], W[i], rr[k].x, dp.x);
+        if (ok[1]) apply<STORAGE, false>(m, D[i + 1], W[i + 1], rr[k].y, dp.y);
+      } else {
+        update_pair(m, D + i, W + i, dp, ok[0], ok[1]);
+      }
+      upd += (ok[0] ? 1u : 0u) + (ok[1] ? 1u : 0u);
+    }
+    return;
   }
+  float fx[4], fy[4], d00[4], d10[4], d01[4], d11[4];
+  bool ok[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float u = __fmul_rn(__fsub_rn(th[i], F.theta_start), F.alpha);
-    const float v = __fmul_rn(__fsub_rn(ph[i], F.phi_start), F.beta);
-    ok[i] = rr[i] > 0.0f;
+    const float rri = (i & 1) ? rr[i >> 1].y : rr[i >> 1].x;
+    const float u = __fmul_rn(__fsub_rn((i & 1) ? th[i >> 1].y : th[i >> 1].x, F.theta_start), F.alpha);
+    const float v = __fmul_rn(__fsub_rn((i & 1) ? ph[i >> 1].y : ph[i >> 1].x, F.phi_start), F.beta);
+    ok[i] = rri > 0.0f;
     d00[i] = d10[i] = d01[i] = d11[i] = 0.0f;
     if (m.lidar_nearest) {
       const float ku = floorf(u), jv = floorf(v);
@@ -1261,6 +1345,7 @@ __device__ __forceinline__ void fuse_lidar(const FrameDev& F, const MapDev& m, c
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     if (!ok[i]) continue;
+    const float rri = (i & 1) ? rr[i >> 1].y : rr[i >> 1].x;
     float d;
     if (m.lidar_nearest) {
       d = d00[i];
@@ -1276,9 +1361,9 @@ __device__ __forceinline__ void fuse_lidar(const FrameDev& F, const MapDev& m, c
       const float bot = __fmaf_rn(fx[i], __fsub_rn(d11[i], d01[i]), d01[i]);
       d = __fmaf_rn(fy[i], __fsub_rn(bot, top), top);
     }
-    const float dp = __fsub_rn(d, rr[i]);
+    const float dp = __fsub_rn(d, rri);
     if (dp < -m.tau) continue;
-    apply<STORAGE, WEIGHTED>(m, D[i], W[i], rr[i], dp);
+    apply<STORAGE, WEIGHTED>(m, D[i], W[i], rri, dp);
     ++upd;
   }
 }
@@ -1448,7 +1533,7 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
         else if (!PINHOLE_ONLY) {
           const int f = __ffs(bits) - 1;  // a LiDAR frame
           bits &= bits - 1u;
-          fuse_lidar<STORAGE, WEIGHTED>(p.fr[f], m, vq, D, W, my_upd);
+          fuse_lidar<STORAGE, WEIGHTED, FAST>(p.fr[f], m, vq, D, W, my_upd);
         }
       }
       Voxels4<STORAGE>::store(m, pool, vq.at, D, W, G4, B);

@@ -216,6 +216,7 @@ bool fast_rcp_ok(const FrameDev& F, double v, int lidar_lsb) {
     if (L2 < -126 || 3.0 * max_rc * max_q + std::fabs((double)F.tloc[2]) >= kTwo126) return false;
     return true;
   }
+  if (F.width > (1 << 21) || F.height > (1 << 21)) return false;  // the kernels' floor of beam coordinates
   const int L = lidar_lsb == INT_MAX ? lsb_m : lsb_m + lidar_lsb;  // beam components are at most 1
   return L >= -126 && 3.0 * max_m * (1.0 + 1e-6) < kTwo126;
 }

@@ -527,7 +527,7 @@ __device__ __forceinline__ void join_exchange(const EsdfDev& e, int nbr, uint32_
 // Three kernels per iteration and a read-back of the set size every four cost
 // the 16 iterations of a room map of 40 frames from scratch and its update
 // after 8 more 470 us of kernels and six host round trips; this launch takes
-// 154 + 75 us.  The sweeps' instructions bound the first phases, the latency
+// 122 + 60 us.  The sweeps' instructions bound the first phases, the latency
 // of a block's dependent steps and of the barriers the small ones.
 __global__ void __launch_bounds__(kLowerThreads, 3)
     esdf_lower_kernel(const MapDev m, const EsdfDev e, uint32_t gen, int with_table) {

@@ -4,15 +4,15 @@
 //  mesh_list_kernel  the blocks to mesh: every block, or every block changed
 //                    since the last extraction together with the seven
 //                    blocks whose cubes reach into it (-x, -y, -z sides)
-//  mesh_kernel       one warp per listed block: the block's 8^3 voxels and
-//                    the +x / +y / +z faces, edges and corner of its
-//                    neighbours (9^3 values) are staged in the warp's part
-//                    of shared memory; each lane classifies two lines of
-//                    eight cubes along x with the case table (held in
-//                    shared memory: lanes index it by their own cases); the
-//                    warp reserves the block's output with one atomic (a
-//                    scan of the lanes' triangle counts), lists the cubes
-//                    with triangles and deals them out across its lanes
+//  mesh_kernel       one warp per listed block: the 9 x 9 rows of nine voxels
+//                    along x that its cubes read (the last of each axis from
+//                    the neighbours) are staged in the warp's part of shared
+//                    memory, the values and per row two 9-bit masks, inside
+//                    and observed; each lane finds the cubes with triangles
+//                    of two lines along x from four rows' masks; the warp
+//                    reserves the block's output with one atomic and emits
+//                    its triangles one per lane, staged so that the stores
+//                    are contiguous
 //
 // A cube joins voxel centres g .. g + (1, 1, 1) and belongs to the block
 // holding g; it is meshed only if its eight corners exist and are observed.
@@ -22,10 +22,10 @@
 namespace gbt {
 namespace {
 
-constexpr int kMeshWarps = 4;                    // blocks meshed at once per CTA
-constexpr int kSide = 9;                         // staged values per axis
-constexpr int kStaged = kSide * kSide * kSide;   // 729
-constexpr int kHalo = kStaged - 512;             // 217 values of the neighbours
+constexpr int kMeshWarps = 4;   // blocks meshed at once per CTA
+constexpr int kRow = 12;        // words per staged row of nine values (16-byte aligned)
+constexpr int kRows = 9 * 9;    // rows (y, z), y fastest
+constexpr int kChunkTris = 32 * 5;  // triangles of 32 cubes, at most
 
 __device__ __forceinline__ int pool_at(const MapDev& m, int x, int y, int z) {
   const int slot = hash_find(m, pack_key(x, y, z));
@@ -56,36 +56,112 @@ __global__ void mesh_list_kernel(const MapDev m, const MeshDev md, int changed_o
   }
 }
 
-// TSDF value of voxel l of pool block q and whether it is observed
-// (W >= min_weight); a missing block (q < 0) is unobserved.
-__device__ __forceinline__ float staged_voxel(const MapDev& m, int q, int l, float min_weight, bool& ok) {
-  ok = false;
-  if (q < 0) return 0.0f;
-  float d, w;
+// TSDF voxel of a storage word: value, and whether it is observed.
+__device__ __forceinline__ void word_voxel(const MapDev& m, uint32_t w, float min_weight, float& d, bool& ok) {
   if (m.storage == kStorageF16) {
-    const __half2 h = reinterpret_cast<const __half2*>(m.pool)[(size_t)q * 512 + l];
+    const __half2 h = *reinterpret_cast<const __half2*>(&w);
     d = __low2float(h) * m.tau;
-    w = __high2float(h);
-  } else if (m.storage == kStorageX16) {
-    const uint32_t word = reinterpret_cast<const uint32_t*>(m.pool)[(size_t)q * 512 + l];
-    d = x16_dist(word, m.x16_unit);
-    w = x16_weight(word);
+    ok = __high2float(h) >= min_weight;
   } else {
-    const float2 v = reinterpret_cast<const float2*>(m.pool)[(size_t)q * 512 + l];
-    d = v.x;
-    w = v.y;
+    d = x16_dist(w, m.x16_unit);
+    ok = x16_weight(w) >= min_weight;
   }
-  ok = w >= min_weight;
-  return d;
 }
 
-__global__ void __launch_bounds__(kMeshWarps * 32, 8)
+// Row r = y + 8 z of pool block q (eight voxels along x) and voxel r of block
+// qx, its first along x, as the row's ninth: values to d, masks returned
+// (inside bits 0 .. 8, observed bits 16 .. 24).  A missing block (negative) is
+// unobserved.
+__device__ __forceinline__ uint32_t load_row(const MapDev& m, int q, int qx, int r, float min_weight, float (&d)[9]) {
+  uint32_t mask = 0u;
+#pragma unroll
+  for (int x = 0; x < 9; ++x) d[x] = 0.0f;
+  if (m.storage == kStorageF32) {
+    if (q >= 0) {
+      const float4* src = reinterpret_cast<const float4*>(m.pool) + (size_t)q * 256 + 4 * r;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4 v = src[k];
+        d[2 * k] = v.x;
+        d[2 * k + 1] = v.z;
+        mask |= (v.y >= min_weight ? 1u << (16 + 2 * k) : 0u) | (v.w >= min_weight ? 2u << (16 + 2 * k) : 0u);
+      }
+    }
+    if (qx >= 0) {
+      const float2 v = reinterpret_cast<const float2*>(m.pool)[(size_t)qx * 512 + 8 * r];
+      d[8] = v.x;
+      mask |= v.y >= min_weight ? 1u << 24 : 0u;
+    }
+  } else {
+    if (q >= 0) {
+      const uint4* src = reinterpret_cast<const uint4*>(m.pool) + (size_t)q * 128 + 2 * r;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const uint4 v = src[k];
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          bool ok;
+          word_voxel(m, w[i], min_weight, d[4 * k + i], ok);
+          mask |= ok ? 1u << (16 + 4 * k + i) : 0u;
+        }
+      }
+    }
+    if (qx >= 0) {
+      bool ok;
+      word_voxel(m, reinterpret_cast<const uint32_t*>(m.pool)[(size_t)qx * 512 + 8 * r], min_weight, d[8], ok);
+      mask |= ok ? 1u << 24 : 0u;
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < 9; ++x) mask |= d[x] < 0.0f ? 1u << x : 0u;
+  return mask;
+}
+
+// One warp's block in shared memory.
+struct MeshBlock {
+  __align__(16) float d[kRow * kRows];  // value at (x, y, z): x + kRow (y + 9 z)
+  uint32_t mask[kRows];
+  uint16_t cube[512];         // the block's cubes with triangles, in order of their lanes
+  uint8_t tri[kChunkTris];    // triangles of 32 cubes: cube in the chunk | number << 5
+  __align__(16) float out[32 * 12];  // 32 triangles' positions, keys or cubes
+};
+
+// Masks of the four rows around line (y, z) of cubes.
+struct LineMasks {
+  uint32_t r0, r1, r2, r3;
+  __device__ __forceinline__ LineMasks(const MeshBlock& b, int y, int z)
+      : r0(b.mask[y + 9 * z]), r1(b.mask[y + 1 + 9 * z]), r2(b.mask[y + 9 * (z + 1)]), r3(b.mask[y + 1 + 9 * (z + 1)]) {}
+  // cubes whose eight corners are observed and not all on one side
+  __device__ __forceinline__ uint32_t surface() const {
+    const uint32_t all = r0 & r1 & r2 & r3, any = r0 | r1 | r2 | r3;
+    const uint32_t both = all & (all >> 1);  // bits 16 ..: observed; bits 0 ..: all corners inside
+    return (both >> 16) & (any | (any >> 1)) & ~both & 0xFFu;
+  }
+  // case of cube x: corner c = x + 2 y + 4 z
+  __device__ __forceinline__ int cube_case(int x) const {
+    return (int)(((r0 >> x) & 3u) | (((r1 >> x) & 3u) << 2) | (((r2 >> x) & 3u) << 4) | (((r3 >> x) & 3u) << 6));
+  }
+};
+
+// Copy a warp's n staged words to out.
+__device__ __forceinline__ void copy_out(const float* stage, float* out, int n, int lane) {
+  __syncwarp();
+  for (int i = lane; i < n; i += 32) __stcs(out + i, stage[i]);
+  __syncwarp();
+}
+
+// Reading every cube's corners and flags one by one (144 shared loads a lane)
+// and storing each lane's triangles a word at a time (24 scattered stores a
+// triangle) took 97.6 us for the blocks of 64 frames of the room; this takes
+// 72.5.  Six CTAs per SM (32 KB of shared memory each) leave a warp about two
+// blocks, so what remains is mostly the latency of a block's chain: list, key,
+// neighbours, rows, reservation, triangles.
+__global__ void __launch_bounds__(kMeshWarps * 32, 6)
     mesh_kernel(const MapDev m, const MeshDev md, const __grid_constant__ MeshTable tab, float min_weight,
                 float* __restrict__ out_pos, int32_t* __restrict__ out_keys,
                 int32_t* __restrict__ out_cube, int64_t cap) {
-  __shared__ float s_d[kMeshWarps][kStaged];         // D at staged (x, y, z), x fastest
-  __shared__ uint8_t s_ok[kMeshWarps][kStaged + 7];  // observed
-  __shared__ uint32_t s_list[kMeshWarps][512];       // the block's cubes with triangles
+  __shared__ MeshBlock s_block[kMeshWarps];
   __shared__ uint8_t s_count[256];
   __shared__ int8_t s_edges[256 * 15];
   {
@@ -95,11 +171,9 @@ __global__ void __launch_bounds__(kMeshWarps * 32, 8)
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* sd = s_d[warp];
-  uint8_t* sok = s_ok[warp];
-  uint32_t* list = s_list[warp];
+  MeshBlock& b = s_block[warp];
   const uint32_t n = (uint32_t)__ldcg(md.cnt);
-  for (uint32_t k = blockIdx.x * kMeshWarps + warp; k < n; k += gridDim.x * kMeshWarps) {
+  for (uint32_t k = warp * gridDim.x + blockIdx.x; k < n; k += gridDim.x * kMeshWarps) {
     const uint32_t p = md.list[k];
     const unsigned long long key = m.block_keys[p];
     const int bx = key_coord(key, 0), by = key_coord(key, 1), bz = key_coord(key, 2);
@@ -107,145 +181,131 @@ __global__ void __launch_bounds__(kMeshWarps * 32, 8)
     // (lane & 1, lane >> 1 & 1, lane >> 2) for lanes 1 .. 7
     const int nbq = lane == 0 ? (int)p
                     : (lane < 8 ? pool_at(m, bx + (lane & 1), by + ((lane >> 1) & 1), bz + (lane >> 2)) : -1);
+    int nb[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) nb[i] = __shfl_sync(0xffffffffu, nbq, i);
     __syncwarp();  // the previous block's reads of the staging are done
+    // rows (y, z) of the block, two per lane; then the rows at y = 8 (lanes
+    // 0 .. 7), z = 8 (lanes 8 .. 15) and both (lane 16)
 #pragma unroll
-    for (int it = 0; it < 16; ++it) {
-      const int l = lane + 32 * it;
-      const int i = (l & 7) + kSide * ((l >> 3) & 7) + kSide * kSide * (l >> 6);
-      bool ok;
-      sd[i] = staged_voxel(m, (int)p, l, min_weight, ok);
-      sok[i] = ok ? 1 : 0;
-    }
-    // the 217 halo values: the +x, +y and +z faces (64 each), the three
-    // edges (8 each) and the corner
-#pragma unroll
-    for (int it = 0; it < (kHalo + 31) / 32; ++it) {
-      const int h = lane + 32 * it;
-      const int a = h & 7, b = (h >> 3) & 7;
-      int nb, sx, sy, sz, l;
-      if (h < 64) {
-        nb = 1; sx = 8; sy = a; sz = b; l = 8 * a + 64 * b;
-      } else if (h < 128) {
-        nb = 2; sx = a; sy = 8; sz = b; l = a + 64 * b;
-      } else if (h < 192) {
-        nb = 4; sx = a; sy = b; sz = 8; l = a + 8 * b;
-      } else if (h < 200) {
-        nb = 3; sx = 8; sy = 8; sz = a; l = 64 * a;
-      } else if (h < 208) {
-        nb = 5; sx = 8; sy = a; sz = 8; l = 8 * a;
-      } else if (h < 216) {
-        nb = 6; sx = a; sy = 8; sz = 8; l = a;
-      } else {
-        nb = 7; sx = 8; sy = 8; sz = 8; l = 0;
+    for (int it = 0; it < 3; ++it) {
+      int q = nb[0], qx = nb[1], r = lane + 32 * it, at = (r & 7) + 9 * (r >> 3);
+      if (it == 2) {
+        q = lane < 8 ? nb[2] : (lane < 16 ? nb[4] : nb[6]);
+        qx = lane < 8 ? nb[3] : (lane < 16 ? nb[5] : nb[7]);
+        r = lane < 8 ? 8 * lane : (lane < 16 ? lane - 8 : 0);
+        at = lane < 8 ? 8 + 9 * lane : (lane < 16 ? lane - 8 + 72 : 80);
+        if (lane > 16) break;
       }
-      const int q = __shfl_sync(0xffffffffu, nbq, nb);
-      if (h < kHalo) {
-        const int i = sx + kSide * sy + kSide * kSide * sz;
-        bool ok;
-        sd[i] = staged_voxel(m, q, l, min_weight, ok);
-        sok[i] = ok ? 1 : 0;
-      }
+      float d[9];
+      const uint32_t mask = load_row(m, q, qx, r, min_weight, d);
+      float4* dst = reinterpret_cast<float4*>(b.d + kRow * at);
+      dst[0] = make_float4(d[0], d[1], d[2], d[3]);
+      dst[1] = make_float4(d[4], d[5], d[6], d[7]);
+      b.d[kRow * at + 8] = d[8];
+      b.mask[at] = mask;
     }
     __syncwarp();
-    // cases of the lane's cubes: lines (y, z) = (lane & 7, lane >> 3) and
-    // (lane & 7, 4 + (lane >> 3)), cubes x = 0 .. 7 along each; a column of
-    // four corners at x gives the even case bits (0, 2, 4, 6) of cube x and
-    // the odd ones of cube x - 1
-    uint32_t cw[4];  // case of cube x of line j in byte x & 3 of cw[2 j + (x >> 2)]
+    // cubes with triangles on the lane's lines (y, z) = (lane & 7, lane >> 3)
+    // and (lane & 7, 4 + (lane >> 3))
     int mine = 0, busy = 0;  // the lane's triangles and cubes with triangles
+    uint32_t surf[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int y = lane & 7, z = (lane >> 3) + 4 * j;
-      const int r = kSide * y + kSide * kSide * z;
-      uint32_t prev_in = 0;
-      bool prev_ok = false;
-      cw[2 * j] = cw[2 * j + 1] = 0u;
-#pragma unroll
-      for (int x = 0; x <= 8; ++x) {
-        const int i0 = r + x, i1 = i0 + kSide, i2 = i0 + kSide * kSide, i3 = i2 + kSide;
-        const uint32_t in = (sd[i0] < 0.0f ? 1u : 0u) | (sd[i1] < 0.0f ? 4u : 0u) | (sd[i2] < 0.0f ? 16u : 0u) |
-                            (sd[i3] < 0.0f ? 64u : 0u);
-        const bool ok = (sok[i0] & sok[i1] & sok[i2] & sok[i3]) != 0;
-        if (x > 0) {
-          const uint32_t ci = (prev_ok && ok) ? (prev_in | (in << 1)) : 0u;
-          cw[2 * j + ((x - 1) >> 2)] |= ci << (8 * ((x - 1) & 3));
-          const int nt = s_count[ci];
-          mine += nt;
-          busy += nt ? 1 : 0;
-        }
-        prev_in = in;
-        prev_ok = ok;
-      }
+      const LineMasks line(b, lane & 7, (lane >> 3) + 4 * j);
+      surf[j] = line.surface();
+      busy += __popc(surf[j]);
+      for (uint32_t w = surf[j]; w; w &= w - 1u) mine += s_count[line.cube_case(__ffs(w) - 1)];
     }
-    // one output reservation per block: inclusive scans of the lanes'
-    // triangle and cube counts
-    int incl = mine, bincl = busy;
+    // one output reservation per block; an inclusive scan of the cube counts
+    const int total = __reduce_add_sync(0xffffffffu, mine);
+    if (total == 0) continue;
+    int incl = busy;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      const int yb = __shfl_up_sync(0xffffffffu, bincl, o);
-      if (lane >= o) {
-        incl += y;
-        bincl += yb;
-      }
+      if (lane >= o) incl += y;
     }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    const int ncubes = __shfl_sync(0xffffffffu, bincl, 31);
+    const int ncubes = __shfl_sync(0xffffffffu, incl, 31);
     unsigned long long base = 0;
-    if (lane == 31 && total) base = atomicAdd(md.cnt + 1, (unsigned long long)total);
-    base = __shfl_sync(0xffffffffu, base, 31);
-    // list the cubes with triangles: cube index (9 bits), case (8 bits),
-    // first triangle within the block (15 bits)
-    {
-      int slot = bincl - busy, tri = incl - mine;
+    if (lane == 0) base = atomicAdd(md.cnt + 1, (unsigned long long)total);
+    int slot = incl - busy;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const int ci = (int)((cw[c >> 2] >> (8 * (c & 3))) & 255u);
-        const int nt = s_count[ci];
-        if (nt) {
-          const int cube = (c & 7) + 8 * (lane & 7) + 64 * ((lane >> 3) + 4 * (c >> 3));
-          list[slot++] = (uint32_t)cube | ((uint32_t)ci << 9) | ((uint32_t)tri << 17);
-          tri += nt;
-        }
-      }
-    }
+    for (int j = 0; j < 2; ++j)
+      for (uint32_t w = surf[j]; w; w &= w - 1u)
+        b.cube[slot++] = (uint16_t)((__ffs(w) - 1) + 8 * (lane & 7) + 64 * ((lane >> 3) + 4 * j));
+    base = __shfl_sync(0xffffffffu, base, 0);
     __syncwarp();
-    // emit: the listed cubes dealt out across the lanes
-    for (int e = lane; e < ncubes; e += 32) {
-      const uint32_t ent = list[e];
-      const int cube = (int)(ent & 511u), ci = (int)((ent >> 9) & 255u);
-      const int x = cube & 7, y = (cube >> 3) & 7, z = cube >> 6;
-      const int nt = s_count[ci];
-      const float* corner = sd + x + kSide * y + kSide * kSide * z;  // corner 0
-      const int gx = 8 * bx + x, gy = 8 * by + y, gz = 8 * bz + z;
-      unsigned long long o = base + (ent >> 17);
-      for (int tr = 0; tr < nt; ++tr, ++o) {
-        if (o >= (unsigned long long)cap) continue;
-        if (out_cube) {
-          out_cube[3 * o] = gx;
-          out_cube[3 * o + 1] = gy;
-          out_cube[3 * o + 2] = gz;
-        }
-        for (int vtx = 0; vtx < 3; ++vtx) {
-          const int ed = s_edges[15 * ci + 3 * tr + vtx];
+    // 32 cubes at a time: their triangles listed, then emitted one per lane
+    for (int e = 0; e < ncubes; e += 32) {
+      int ent = 0, nt = 0;  // this lane's cube | case << 9, and its triangles
+      if (e + lane < ncubes) {
+        const int c = b.cube[e + lane];
+        const LineMasks line(b, (c >> 3) & 7, c >> 6);
+        const int ci = line.cube_case(c & 7);
+        ent = c | (ci << 9);
+        nt = s_count[ci];
+      }
+      int end = nt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += y;
+      }
+      const int tris = __shfl_sync(0xffffffffu, end, 31);
+      for (int i = 0; i < nt; ++i) b.tri[end - nt + i] = (uint8_t)(lane | (i << 5));
+      __syncwarp();
+      for (int t0 = 0; t0 < tris; t0 += 32) {
+        const int code = t0 + lane < tris ? b.tri[t0 + lane] : 0;
+        const int te = __shfl_sync(0xffffffffu, ent, code & 31);
+        const int cube = te & 511, ci = te >> 9, tr = code >> 5;
+        const int x = cube & 7, y = (cube >> 3) & 7, z = cube >> 6;
+        const int gx = 8 * bx + x, gy = 8 * by + y, gz = 8 * bz + z;
+        const float* corner = b.d + x + kRow * (y + 9 * z);  // corner 0
+        int g[3][3], axes[3];
+        float* o = b.out + 9 * lane;
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          const int ed = s_edges[15 * ci + 3 * tr + v];
           const int axis = ed >> 2, u = ed & 1, w = (ed >> 1) & 1;
           // lower corner of edge ed: bit `axis` clear, the other two axes u, w
           const int o1 = axis == 0 ? 1 : 0, o2 = axis == 2 ? 1 : 2;
-          const int lo = (u << o1) | (w << o2), hi = lo | (1 << axis);
-          const float dlo = corner[(lo & 1) + kSide * ((lo >> 1) & 1) + kSide * kSide * (lo >> 2)];
-          const float dhi = corner[(hi & 1) + kSide * ((hi >> 1) & 1) + kSide * kSide * (hi >> 2)];
+          const int lo = (u << o1) | (w << o2);
+          const float* c0 = corner + (lo & 1) + kRow * (((lo >> 1) & 1) + 9 * (lo >> 2));
+          const float dlo = c0[0], dhi = c0[axis == 0 ? 1 : (axis == 1 ? kRow : 9 * kRow)];
           const float tt = __fdiv_rn(dlo, __fsub_rn(dlo, dhi));
-          const int g[3] = {gx + (lo & 1), gy + ((lo >> 1) & 1), gz + (lo >> 2)};
+          g[v][0] = gx + (lo & 1);
+          g[v][1] = gy + ((lo >> 1) & 1);
+          g[v][2] = gz + (lo >> 2);
+          axes[v] = axis;
 #pragma unroll
           for (int a = 0; a < 3; ++a) {
-            float cf = __fadd_rn((float)g[a], 0.5f);
+            float cf = __fadd_rn((float)g[v][a], 0.5f);
             if (a == axis) cf = __fadd_rn(cf, tt);
-            out_pos[9 * o + 3 * vtx + a] = __fmul_rn(cf, m.v);
-            if (out_keys) out_keys[12 * o + 4 * vtx + a] = g[a];
+            o[3 * v + a] = __fmul_rn(cf, m.v);
           }
-          if (out_keys) out_keys[12 * o + 4 * vtx + 3] = axis;
         }
+        // the 32 triangles' words are contiguous in each output
+        const long long room = (long long)cap - (long long)base;
+        const int count = (int)max(0ll, min((long long)min(32, tris - t0), room));
+        copy_out(b.out, out_pos + 9 * base, 9 * count, lane);
+        if (out_keys) {
+          int* ko = reinterpret_cast<int*>(b.out) + 12 * lane;
+#pragma unroll
+          for (int v = 0; v < 3; ++v)
+            *reinterpret_cast<int4*>(ko + 4 * v) = make_int4(g[v][0], g[v][1], g[v][2], axes[v]);
+          copy_out(b.out, reinterpret_cast<float*>(out_keys) + 12 * base, 12 * count, lane);
+        }
+        if (out_cube) {
+          int* co = reinterpret_cast<int*>(b.out) + 3 * lane;
+          co[0] = gx;
+          co[1] = gy;
+          co[2] = gz;
+          copy_out(b.out, reinterpret_cast<float*>(out_cube) + 3 * base, 3 * count, lane);
+        }
+        base += (unsigned long long)min(32, tris - t0);
       }
+      __syncwarp();  // the chunk's triangle list is used up
     }
   }
 }
@@ -264,7 +324,7 @@ cudaError_t launch_mesh(const MapDev& m, const MeshDev& md, const MeshTable& tab
                         int64_t cap, cudaStream_t s) {
   const int sms = sm_count();
   mesh_list_kernel<<<sms * 2, 256, 0, s>>>(m, md, changed_only, gen);
-  mesh_kernel<<<sms * 8, kMeshWarps * 32, 0, s>>>(m, md, table, min_weight, pos, keys, cubes, cap);
+  mesh_kernel<<<sms * 6, kMeshWarps * 32, 0, s>>>(m, md, table, min_weight, pos, keys, cubes, cap);
   return cudaGetLastError();
 }
 

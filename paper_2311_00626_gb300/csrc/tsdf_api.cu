@@ -435,6 +435,7 @@ void free_map(tsdf_map* m) {
     cudaFree(m->mesh.list);
     cudaFree(m->mesh.stamp);
     cudaFree(m->mesh.cnt);
+    cudaFreeHost(m->mesh.host);
   }
   if (m->esdf_on) {
     cudaFree(m->esdf.st);
@@ -1362,20 +1363,21 @@ tsdf_status map_mesh(tsdf_map* map, float min_weight, int32_t changed_only, floa
     if (cudaMalloc(&md.list, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
         cudaMalloc(&md.stamp, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
         cudaMalloc(&md.cnt, sizeof(unsigned long long) * 2) != cudaSuccess ||
+        cudaMallocHost(&md.host, sizeof(unsigned long long) * 2) != cudaSuccess ||
         cudaMemset(md.stamp, 0, sizeof(uint32_t) * map->max_blocks) != cudaSuccess)
       return cuda_fail();
     map->mesh_gen = 0;
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  unsigned long long cnt[2] = {0, 0};
-  if (cudaMemsetAsync(md.cnt, 0, sizeof(cnt), s) != cudaSuccess ||
+  if (cudaMemsetAsync(md.cnt, 0, sizeof(unsigned long long) * 2, s) != cudaSuccess ||
       gbt::launch_mesh(map->dev, md, mesh_table(), changed_only ? 1 : 0, ++map->mesh_gen, min_weight,
                        tri_pos_dev, tri_keys_dev, tri_cube_dev, cap, s) != cudaSuccess ||
-      cudaMemcpyAsync(cnt, md.cnt, sizeof(cnt), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(md.host, md.cnt, sizeof(unsigned long long) * 2, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail();
-  *n_tris = (int64_t)cnt[1];
-  return cnt[1] > (unsigned long long)cap ? TSDF_ERR_CAPACITY : TSDF_OK;
+  const unsigned long long tris = md.host[1];
+  *n_tris = (int64_t)tris;
+  return tris > (unsigned long long)cap ? TSDF_ERR_CAPACITY : TSDF_OK;
 }
 
 tsdf_status map_wait_test(tsdf_map* map, int32_t extra_ctas) {

@@ -263,7 +263,7 @@ cudaError_t launch_dependent(void (*k)(P...), unsigned blocks, unsigned threads,
 // pool index, and the other points' probes are all issued before any is
 // used.  One point per thread waited on point -> key -> slot -> value chains:
 // 5.9 M voxel centres of a 5 cm map 41.5 us, four per thread 26.1 us (28
-// bytes a point; the 300-frame room's 10 M points 95 -> 63 us).
+// bytes a point; the 300-frame room's 10 M points 95 -> 57 us).
 constexpr int kPointsPerThread = 4;
 
 // Quotients of the points by the voxel edge, rounded to nearest as x / v is:
@@ -409,6 +409,7 @@ struct MeshDev {
   uint32_t* list;     // [max_blocks] blocks to mesh
   uint32_t* stamp;    // [max_blocks] generation that listed the block
   unsigned long long* cnt;  // [0] list size, [1] triangles produced
+  unsigned long long* host; // pinned copy of cnt
 };
 cudaError_t launch_mesh(const MapDev& m, const MeshDev& md, const MeshTable& table, int changed_only,
                         uint32_t gen, float min_weight, float* pos, int32_t* keys, int32_t* cubes,

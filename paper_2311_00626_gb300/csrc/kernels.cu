@@ -1941,7 +1941,11 @@ cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int per_sm, cudaStrea
 #define GBT_INTEG(ST, PH) \
   (fast ? launch_variant<NF, NM, ST, PH, false, true>(p, per_sm, limit, s) \
         : launch_variant<NF, NM, ST, PH, false, false>(p, per_sm, limit, s))
-#define GBT_WEIGHTED(ST) launch_variant<NF, NM, ST, false, true, false>(p, per_sm, limit, s)
+  // weighted maps: pinhole batches with fast reciprocals leave the LiDAR code
+  // and the IEEE reciprocals out too (24 frames of 1280x720: 39.0 -> 34.2 us)
+#define GBT_WEIGHTED(ST) \
+  (ph && fast ? launch_variant<NF, NM, ST, true, true, true>(p, per_sm, limit, s) \
+              : launch_variant<NF, NM, ST, false, true, false>(p, per_sm, limit, s))
   if (st == kStorageColor) return GBT_INTEG(kStorageColor, true);
   if (st == kStorageOcc) return ph ? GBT_INTEG(kStorageOcc, true) : GBT_INTEG(kStorageOcc, false);
   if (st == kStorageX16) {

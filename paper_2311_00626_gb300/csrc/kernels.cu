@@ -14,11 +14,11 @@
 //                     where a conservative test cannot show that their
 //                     blocks are known already.
 //  integrate_kernel   Sec. IV-B second step (Eq. 1-3 and the update
-//                     functors: TSDF, occupancy, colour): persistent CTAs
-//                     take work-list blocks, 4 voxels per thread held in
-//                     registers across every frame of the batch that met the
-//                     block, one coalesced read and write per block and
-//                     batch.
+//                     functors: TSDF, occupancy, colour): the warps of a
+//                     persistent grid take quarters of work-list blocks, 4
+//                     voxels per thread held in registers across every frame
+//                     of the batch that met the block, one coalesced read
+//                     and write per block and batch.
 //  query_kernel,      point -> voxel lookup through the hash.
 //  query_color_kernel
 //  decay_kernel       occupancy decay over every allocated block (Sec. V-E).

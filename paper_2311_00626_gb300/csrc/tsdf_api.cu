@@ -47,6 +47,7 @@ struct tsdf_map {
   // further mask / work-list / control sets: with them the allocation of
   // sub-batches runs on `aux` while earlier ones integrate
   gbt::MoreSets more;
+  char* more_base;  // their one allocation
   cudaStream_t aux;
   cudaEvent_t ev_alloc[4], ev_int[4], ev_start;
   // host-input batches: copy stream and per-sub-batch copy events (lazy)
@@ -425,11 +426,7 @@ tsdf_status read_counters(const tsdf_map* m, unsigned long long c[gbt::kNumCount
 }
 
 void free_map(tsdf_map* m) {
-  for (int k = 0; k < gbt::kSets - 1; ++k) {
-    cudaFree(m->more.mask[k]);
-    cudaFree(m->more.list[k]);
-    cudaFree(m->more.ctl[k]);
-  }
+  cudaFree(m->more_base);
   cudaFree(m->dev.dirty);
   if (m->mesh_on) {
     cudaFree(m->mesh.list);
@@ -573,10 +570,16 @@ tsdf_status map_create_ex(float voxel_size, int32_t truncation_voxels, float max
   for (int i = 0; ok && i < 4; ++i)
     ok = cudaEventCreateWithFlags(&m->ev_alloc[i], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&m->ev_int[i], cudaEventDisableTiming) == cudaSuccess;
-  for (int k = 0; ok && k < gbt::kSets - 1; ++k)
-    ok = cudaMalloc(&m->more.mask[k], sizeof(uint32_t) * cap) == cudaSuccess &&
-         cudaMalloc(&m->more.list[k], sizeof(uint32_t) * o.max_blocks) == cudaSuccess &&
-         cudaMalloc(&m->more.ctl[k], sizeof(unsigned int) * 4) == cudaSuccess;
+  // the further work sets in one allocation
+  const size_t mask_bytes = ((size_t)cap * 4 + 255) / 256 * 256, list_bytes = ((size_t)o.max_blocks * 4 + 255) / 256 * 256;
+  const size_t set_bytes = mask_bytes + list_bytes + 256;
+  ok = ok && cudaMalloc(&m->more_base, set_bytes * (gbt::kSets - 1)) == cudaSuccess;
+  for (int k = 0; ok && k < gbt::kSets - 1; ++k) {
+    char* base = m->more_base + k * set_bytes;
+    m->more.mask[k] = reinterpret_cast<uint32_t*>(base);
+    m->more.list[k] = reinterpret_cast<uint32_t*>(base + mask_bytes);
+    m->more.ctl[k] = reinterpret_cast<unsigned int*>(base + mask_bytes + list_bytes);
+  }
   if (ok)
     ok = gbt::launch_reset(d, m->cap, m->more, 0) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;

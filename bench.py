@@ -561,8 +561,8 @@ def main():
             "roofline": {"bound": "alu", "achieved": alloc_achieved / 1e12,
                          "peak": ALU_PEAK_OPS / 1e12, "unit": "Tops/s",
                          "frac": alloc_achieved / ALU_PEAK_OPS,
-                         "traffic": _traffic("band_alloc_kernel"),
-                         "kernel": "band_alloc_kernel", "share_of_kernel_time": alloc_share,
+                         "traffic": _traffic("patch_alloc_kernel"),
+                         "kernel": "patch_alloc_kernel", "share_of_kernel_time": alloc_share,
                          "peak_source": "152 SMs x 128 lanes x 2070 MHz",
                          "ops_per_launch": alloc_ops_per_launch,
                          "ms_per_launch": alloc_ms_per_launch,
@@ -863,8 +863,7 @@ def bench_layers(args):
         return {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                 "bytes": nbytes, "peak_source": hbm_src}
 
-    def esdf_launches(iters):  # mark, clear, neighbours; four 3-kernel iterations per check
-        return 3 + 12 * max(1, -(-iters // 4))
+    esdf_launches = 3  # mark, clear, and every lowering iteration in one
     # the mesh lists every block whose cubes reach into a changed block, up
     # to eight per changed block; the changed blocks bound it from below
     rl = {
@@ -889,8 +888,7 @@ def bench_layers(args):
             "ms": t, "triangles": {"full": last["tris_full"], "incremental": last["tris_inc"]},
             "esdf": {"full": last["full"], "incremental": last["inc"]},
             "roofline": rl,
-            "gpu_launches": args.steps * (esdf_launches(last["full"]["iterations"])
-                                          + esdf_launches(last["inc"]["iterations"]) + 2 * 2),
+            "gpu_launches": args.steps * (2 * esdf_launches + 2 * 2),
         }), flush=True)
     m.close()
 

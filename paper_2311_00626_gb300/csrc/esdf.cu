@@ -661,6 +661,9 @@ __global__ void esdf_reset_kernel(const MapDev m, const EsdfDev e) {
   uint4* st = reinterpret_cast<uint4*>(e.st);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     st[i] = make_uint4(0u, 0u, 0u, 0u);
+  // an update that gave up at a barrier leaves blocks in their second buffer
+  for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n / 128; p += (size_t)gridDim.x * blockDim.x)
+    e.ver[p] = 0u;
   if (blockIdx.x == 0 && threadIdx.x < 4) e.stats[threadIdx.x] = 0ull;
 }
 

@@ -63,6 +63,7 @@ struct tsdf_map {
   tsdf_esdf_opts esdf_opts;
   uint32_t esdf_gen;      // generation of the last update set / tlist built
   uint32_t* esdf_host;    // pinned copy of esdf.cnt
+  bool esdf_broken;       // an update gave up at a barrier
   // meshing scratch, allocated by the first map_mesh
   bool mesh_on;
   gbt::MeshDev mesh;
@@ -1166,6 +1167,7 @@ tsdf_status map_esdf_update(tsdf_map* map, const tsdf_esdf_opts* opts, void* cud
   if (!(o.site_eps >= 0.0f) || !std::isfinite(o.site_eps) || !std::isfinite(o.min_weight) ||
       o.max_dist_vox < 1 || o.max_dist_vox > 255)
     return TSDF_ERR_ARG;
+  if (map->esdf_broken) return TSDF_ERR_TIMEOUT;  // until map_reset
   if (map->esdf_on && (o.site_eps != map->esdf_opts.site_eps ||
                        o.min_weight != map->esdf_opts.min_weight ||
                        o.max_dist_vox != map->esdf_opts.max_dist_vox))
@@ -1190,6 +1192,7 @@ tsdf_status map_esdf_update(tsdf_map* map, const tsdf_esdf_opts* opts, void* cud
   map->esdf_gen = g + 1 + map->esdf_host[gbt::kEcIterations];
   if (map->esdf_host[gbt::kEcTimeout]) {  // a grid barrier gave up: the layer is not converged
     map->status_seen |= gbt::kStTimeout;
+    map->esdf_broken = true;
     return TSDF_ERR_TIMEOUT;
   }
   return TSDF_OK;
@@ -1396,6 +1399,7 @@ tsdf_status map_reset(tsdf_map* map, void* cuda_stream) {
   if (map->esdf_on && gbt::launch_esdf_reset(map->dev, map->esdf, s) != cudaSuccess) return cuda_fail();
   if (gbt::launch_reset(map->dev, map->cap, map->more, s) != cudaSuccess) return cuda_fail();
   map->status_seen = 0;
+  map->esdf_broken = false;
   map->frames = 0;
   return TSDF_OK;
 }

@@ -434,12 +434,13 @@ tsdf_status map_mesh(tsdf_map* map, float min_weight, int32_t changed_only, floa
                      int32_t* tri_keys_dev, int32_t* tri_cube_dev, int64_t cap, int64_t* n_tris,
                      void* cuda_stream);
 
-/* map_wait_test — test hook for the bounded wait of TSDF_LAUNCH_FUSED:
- * while extra_ctas > 0, the map's fused launches wait at their grid-wide
- * barrier for extra_ctas more CTAs than they have, so the wait runs out
- * after about a second, the launch skips its integration and the map
- * reports TSDF_ERR_TIMEOUT (cleared by map_reset).  0 restores normal
- * operation.  TSDF_ERR_ARG for a negative count. */
+/* map_wait_test — test hook for the bounded device waits: while
+ * extra_ctas > 0, the map's fused launches (TSDF_LAUNCH_FUSED) wait at their
+ * grid-wide barrier for extra_ctas more CTAs than they have, so the wait runs
+ * out after about a second, the launch skips its integration and the map
+ * reports TSDF_ERR_TIMEOUT (cleared by map_reset).  An ESDF update waits the
+ * same way at its fifth grid-wide barrier, if it needs that many.  0 restores
+ * normal operation.  TSDF_ERR_ARG for a negative count. */
 tsdf_status map_wait_test(tsdf_map* map, int32_t extra_ctas);
 
 /* map_reset — drop every block (keeps the allocation), enqueued on

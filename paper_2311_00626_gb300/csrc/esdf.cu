@@ -431,8 +431,11 @@ struct LowerBlock {
 
 // Grid-wide barrier `k` (0, 1, ...) of a cooperative launch: every CTA is
 // resident, so the wait ends; after a second of the global timer it gives up
-// all the same, flags it and returns false to the whole CTA.
-__device__ __forceinline__ bool grid_barrier(const EsdfDev& e, unsigned k, bool* s_ok) {
+// all the same, flags it and returns false to the whole CTA.  extra (a test
+// hook): from barrier kWaitTestBarrier on, CTAs expected that do not exist.
+constexpr unsigned kWaitTestBarrier = 4;  // after phase 3: a few exchange generations are stamped
+__device__ __forceinline__ bool grid_barrier(const EsdfDev& e, unsigned k, unsigned extra, bool* s_ok) {
+  const unsigned expected = (k + 1u) * gridDim.x + (k >= kWaitTestBarrier ? extra : 0u);
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -443,7 +446,7 @@ __device__ __forceinline__ bool grid_barrier(const EsdfDev& e, unsigned k, bool*
     for (;;) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(e.cnt + kEcBarrier) : "memory");
-      if (v >= (k + 1u) * gridDim.x) break;
+      if (v >= expected) break;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
       if (t - t0 > 1000000000ull) {
         ok = false;
@@ -530,7 +533,7 @@ __device__ __forceinline__ void join_exchange(const EsdfDev& e, int nbr, uint32_
 // 122 + 60 us.  The sweeps' instructions bound the first phases, the latency
 // of a block's dependent steps and of the barriers the small ones.
 __global__ void __launch_bounds__(kLowerThreads, 3)
-    esdf_lower_kernel(const MapDev m, const EsdfDev e, uint32_t gen, int with_table) {
+    esdf_lower_kernel(const MapDev m, const EsdfDev e, uint32_t gen, int with_table, unsigned wait_extra) {
   __shared__ LowerBlock blocks[kLowerWarps];
   __shared__ bool s_ok;
   const int lane = threadIdx.x & 31;
@@ -543,7 +546,7 @@ __global__ void __launch_bounds__(kLowerThreads, 3)
   unsigned barrier = 0;
   if (with_table) {
     neighbour_table(m, e);
-    if (!grid_barrier(e, barrier++, &s_ok)) return;
+    if (!grid_barrier(e, barrier++, wait_extra, &s_ok)) return;
   }
   const uint32_t my_face = lane < 6 ? (uint32_t)lane : 0u;
   // phase 0: sweep the update set in place
@@ -559,7 +562,7 @@ __global__ void __launch_bounds__(kLowerThreads, 3)
   }
   uint32_t swept = n0, pulled = 0, k = 1;
   for (;; ++k) {
-    if (!grid_barrier(e, barrier++, &s_ok)) return;
+    if (!grid_barrier(e, barrier++, wait_extra, &s_ok)) return;
     const uint32_t n = __ldcg(e.cnt + kEcExchange + k % 3);
     if (n == 0) break;
     const uint32_t* list = (k & 1u) ? e.tlist[1] : e.tlist[0];
@@ -655,15 +658,16 @@ __global__ void __launch_bounds__(kLowerThreads, 3)
 // Only the map's own blocks have states (a pool block gets its first ones when
 // it is marked, after it was handed out), so a reset clears those and not the
 // whole pool: 128 MiB for 2^16 pool blocks, about 25 us, of which a room fills
-// a tenth.
+// a tenth.  An update that gave up at a barrier leaves more behind: blocks in
+// their second buffer, and stamps of generations that the host never learned
+// of and will give out again.
 __global__ void esdf_reset_kernel(const MapDev m, const EsdfDev e) {
   const size_t n = (size_t)n_blocks(m) * 128;
   uint4* st = reinterpret_cast<uint4*>(e.st);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     st[i] = make_uint4(0u, 0u, 0u, 0u);
-  // an update that gave up at a barrier leaves blocks in their second buffer
   for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n / 128; p += (size_t)gridDim.x * blockDim.x)
-    e.ver[p] = 0u;
+    e.ver[p] = e.stamp_s[p] = e.stamp_t[p] = 0u;
   if (blockIdx.x == 0 && threadIdx.x < 4) e.stats[threadIdx.x] = 0ull;
 }
 
@@ -789,8 +793,9 @@ cudaError_t launch_esdf_reset(const MapDev& m, const EsdfDev& e, cudaStream_t s)
 
 // The lowering iterations, launched cooperatively with every CTA that can be
 // resident.  Exchange generations start at gen.  The neighbour table is built
-// here unless the mark stage of an occupancy layer built it.
-cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s) {
+// here unless the mark stage of an occupancy layer built it.  wait_extra: the
+// barriers' test hook.
+cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, unsigned wait_extra, cudaStream_t s) {
   static std::atomic<int> fit{0};  // resident CTAs per SM (all devices are alike here)
   int n = fit.load(std::memory_order_relaxed);
   if (n == 0) {
@@ -808,7 +813,7 @@ cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, c
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, esdf_lower_kernel, m, e, gen, m.storage == kStorageOcc ? 0 : 1);
+  return cudaLaunchKernelEx(&cfg, esdf_lower_kernel, m, e, gen, m.storage == kStorageOcc ? 0 : 1, wait_extra);
 }
 
 cudaError_t launch_esdf_query(const MapDev& m, const EsdfDev& e, const float* pts, int64_t n,

@@ -40,7 +40,7 @@ struct tsdf_map {
   int integrate_per_sm;  // integration CTAs per SM, 0 = as many as fit
   int tile_h;  // allocation tile height, 0 = automatic
   int launch_mode;     // TSDF_LAUNCH_SPLIT or TSDF_LAUNCH_FUSED
-  int32_t wait_extra;  // map_wait_test: extra CTAs the fused launch's grid-wide wait expects
+  int32_t wait_extra;  // map_wait_test: CTAs that bounded waits expect and that do not exist
   int64_t frames;
   unsigned long long status_seen;  // device status bits observed by the host
   std::vector<LidarTable> tables;
@@ -1185,7 +1185,7 @@ tsdf_status map_esdf_update(tsdf_map* map, const tsdf_esdf_opts* opts, void* cud
       gbt::launch_esdf_mark(map->dev, e, g, s) != cudaSuccess ||
       gbt::launch_esdf_clear(map->dev, e, g, s) != cudaSuccess ||
       // lower until no block changes, in one launch
-      gbt::launch_esdf_lower(map->dev, e, g + 1, s) != cudaSuccess)
+      gbt::launch_esdf_lower(map->dev, e, g + 1, (unsigned)map->wait_extra, s) != cudaSuccess)
     return cuda_fail();
   tsdf_status st = esdf_read_counts(map, s);
   if (st != TSDF_OK) return st;

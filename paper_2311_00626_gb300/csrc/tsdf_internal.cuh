@@ -393,7 +393,7 @@ cudaError_t launch_esdf_reset(const MapDev& m, const EsdfDev& e, cudaStream_t s)
 // ESDF stages (esdf.cu).
 cudaError_t launch_esdf_mark(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);
 cudaError_t launch_esdf_clear(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);
-cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, cudaStream_t s);
+cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, unsigned wait_extra, cudaStream_t s);
 cudaError_t launch_esdf_query(const MapDev& m, const EsdfDev& e, const float* pts, int64_t n,
                               float* dist, cudaStream_t s);
 cudaError_t launch_import(const MapDev& m, const int32_t* keys, const float* D, const float* W,

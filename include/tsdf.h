@@ -388,7 +388,8 @@ typedef struct {
  * blocks marked are the changed ones and their face neighbours, and a
  * map_decay_occupancy call counts as a change of every block it alters.
  * Enqueued on cuda_stream; waits for the stream.  TSDF_ERR_TIMEOUT if a
- * bounded device wait gave up, and from later calls of it until map_reset.
+ * bounded device wait gave up: the layer is then half done, and later updates,
+ * map_esdf_query and map_esdf_export return TSDF_ERR_TIMEOUT until map_reset.
  */
 tsdf_status map_esdf_update(tsdf_map* map, const tsdf_esdf_opts* opts, void* cuda_stream);
 

@@ -1213,6 +1213,7 @@ tsdf_status map_esdf_stats(const tsdf_map* map, int64_t out[4]) {
 
 tsdf_status map_esdf_export(const tsdf_map* map, int32_t* keys_host, uint32_t* states_host, int64_t n) {
   if (!map || !keys_host || !map->esdf_on) return TSDF_ERR_ARG;
+  if (map->esdf_broken) return TSDF_ERR_TIMEOUT;  // half-done states, some in the other buffer
   int64_t nb = 0;
   tsdf_status st = map_num_blocks(map, &nb);
   if (st != TSDF_OK) return st;
@@ -1249,6 +1250,7 @@ tsdf_status map_esdf_query(const tsdf_map* map, const float* pts_dev, int64_t n,
                            void* cuda_stream) {
   if (!map || !map->esdf_on || n < 0 || (n > 0 && (!pts_dev || !dist_dev))) return TSDF_ERR_ARG;
   if (!on_device(map)) return TSDF_ERR_STATE;
+  if (map->esdf_broken) return TSDF_ERR_TIMEOUT;
   if (gbt::launch_esdf_query(map->dev, map->esdf, pts_dev, n, dist_dev, (cudaStream_t)cuda_stream) !=
       cudaSuccess)
     return cuda_fail();

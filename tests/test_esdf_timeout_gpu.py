@@ -58,3 +58,25 @@ def test_reset_restores_the_layer_after_an_update_gave_up():
         g.reset()
     g.close()
     o.close()
+
+
+def test_a_half_done_layer_is_not_read_out():
+    """Between the update that gave up and the reset, the states are a mix of
+    two buffers and of iterations: reading them is refused."""
+    blocks = _wall()
+    g = gt.TsdfMap(EPS, max_blocks=1 << 12)
+    g.import_blocks(*blocks)
+    g.esdf_update(EPS, 1e-4, RANGE)
+    pts = torch.from_numpy(((blocks[0] * 8 + 4.5) * EPS).astype(np.float32)).cuda()
+    dist = torch.empty(len(pts), device="cuda")
+    g.reset()
+    _gave_up(g, blocks)
+    for call in (lambda: g.esdf_query(pts, dist), g.esdf_export, lambda: g.esdf_update(EPS, 1e-4, RANGE)):
+        with pytest.raises(gt.TsdfError) as e:
+            call()
+        assert e.value.code == TIMEOUT
+    g.reset()
+    assert len(g.esdf_export()[0]) == 0
+    g.esdf_query(pts, dist)
+    assert torch.isnan(dist).all()
+    g.close()

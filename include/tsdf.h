@@ -439,9 +439,12 @@ tsdf_status map_mesh(tsdf_map* map, float min_weight, int32_t changed_only, floa
  * extra_ctas > 0, the map's fused launches (TSDF_LAUNCH_FUSED) wait at their
  * grid-wide barrier for extra_ctas more CTAs than they have, so the wait runs
  * out after about a second, the launch skips its integration and the map
- * reports TSDF_ERR_TIMEOUT (cleared by map_reset).  An ESDF update waits the
- * same way at its fifth grid-wide barrier, if it needs that many.  0 restores
- * normal operation.  TSDF_ERR_ARG for a negative count. */
+ * reports TSDF_ERR_TIMEOUT (cleared by map_reset).  Split integration
+ * launches find no work-list entry published and give up after some 0.1 s:
+ * every map of the call reports TSDF_ERR_TIMEOUT (the first map's hook
+ * counts).  An ESDF update waits at its fifth grid-wide barrier, if it needs
+ * that many.  0 restores normal operation.  TSDF_ERR_ARG for a negative
+ * count. */
 tsdf_status map_wait_test(tsdf_map* map, int32_t extra_ctas);
 
 /* map_reset — drop every block (keeps the allocation), enqueued on

@@ -322,8 +322,8 @@ def map_walk_stats(m: int, enable: bool = True):
 
 def map_wait_test(m: int, extra_ctas: int):
     """Test hook: fused launches and ESDF updates wait for extra_ctas CTAs that
-    do not exist (their bounded wait runs out: TSDF_ERR_TIMEOUT); 0 restores
-    them."""
+    do not exist, split integrations for an entry that is never published
+    (their bounded waits run out: TSDF_ERR_TIMEOUT); 0 restores them."""
     _check(lib().map_wait_test(m, int(extra_ctas)), "map_wait_test")
 
 

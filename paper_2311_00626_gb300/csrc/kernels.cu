@@ -1413,9 +1413,10 @@ __device__ __forceinline__ T meta_load(const T* a) {
 // next entry (handed out dynamically: blocks differ in their frame counts)
 // into a ring of kRing slots; a slot is free once the four slabs of its last
 // entry are done.  Tickets go out in order and an entry's slabs depend on no
-// later one, so both waits end; they are bounded all the same.  The warp that
-// finishes an entry's last slab clears its mask (every slab has read it by
-// then).  The last CTA to finish resets every map's work list.
+// later one, so both waits end; they are bounded all the same (BatchParams::
+// wait_extra withholds the first entry to see that).  The warp that finishes
+// an entry's last slab clears its mask (every slab has read it by then).  The
+// last CTA to finish resets every map's work list.
 template <int NF, int NM, bool COHERENT, int STORAGE, bool PINHOLE_ONLY, bool WEIGHTED, bool FAST>
 __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, IntegSmem<NF, NM>& sm,
                                                   bool wait) {
@@ -1423,7 +1424,7 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
   for (int f = threadIdx.x; f < p.n_frames; f += blockDim.x)
     if (p.fr[f].kind == kSensorPinhole) stage_frame(p.fr[f], sm.fp[f]);
   if (threadIdx.x < kRing) {
-    sm.seq[threadIdx.x] = threadIdx.x ? 0xFFFFFFFFu : 0u;
+    sm.seq[threadIdx.x] = threadIdx.x || p.wait_extra ? 0xFFFFFFFFu : 0u;
     sm.entry[threadIdx.x] = blockIdx.x;
     sm.done[threadIdx.x] = 0u;
   }
@@ -1497,7 +1498,9 @@ __device__ __forceinline__ void integrate_entries(const BatchParams<NF, NM>& p, 
       *(volatile uint32_t*)&sm.seq[next % kRing] = next;
     }
     if (!__all_sync(0xffffffffu, ok)) {
-      if (lane == 0) atomicOr(p.maps[0].counters + kCntStatus, (unsigned long long)kStTimeout);
+      // some of the batch's entries are left out, whichever map they are in
+      if (lane == 0)
+        for (int i = 0; i < p.n_maps; ++i) atomicOr(p.maps[i].counters + kCntStatus, (unsigned long long)kStTimeout);
       break;
     }
     if (!work) break;

@@ -394,6 +394,7 @@ tsdf_status integrate_one(tsdf_map* m, int kind, const tsdf_pinhole* ph, const t
   p.n_frames = 1;
   p.n_maps = 1;
   p.maps[0] = m->dev;
+  p.wait_extra = m->wait_extra;
   tsdf_status st = fill_frame(m, 0, kind, ph, li, depth, rgba, T, p.fr[0]);
   if (st != TSDF_OK) return st;
   p.fr[0].bit = 0;
@@ -737,6 +738,7 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
     std::memset(&p, 0, sizeof(p));
     p.n_frames = nf;
     p.n_maps = n_maps;
+    p.wait_extra = lead->wait_extra;
     for (int i = 0; i < n_maps; ++i) p.maps[i] = view_set(maps[i], piped ? b % gbt::kSets : 0);
     p.fast_rcp = 1;
     for (int f = 0; f < nf; ++f) {
@@ -751,6 +753,7 @@ tsdf_status run_batch(tsdf_map* const* maps, int32_t n_maps, std::vector<FrameDe
     if (n_maps == 1) {
       p1.n_frames = p.n_frames;
       p1.n_maps = 1;
+      p1.wait_extra = p.wait_extra;
       p1.fast_rcp = p.fast_rcp;
       p1.maps[0] = p.maps[0];
       std::memcpy(p1.fr, p.fr, sizeof(p.fr));

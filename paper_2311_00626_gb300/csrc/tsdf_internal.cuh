@@ -186,7 +186,8 @@ struct BatchParams {
   int32_t n_maps;
   int32_t overlap;     // launched as a programmatic dependent of the stream's previous kernel
   int32_t alloc_ctas;  // allocation tiles of the batch (the fused kernel loops over them)
-  int32_t wait_extra;  // test hook: the fused kernel's grid wait expects this many extra CTAs
+  int32_t wait_extra;  // test hook: the fused kernel's grid wait expects this many extra CTAs; in an
+                       // integration launch, if not 0, no warp gets an entry
   int32_t fast_rcp;    // every reciprocal of the batch's decisions lies in [2^-126, 2^126] or is not taken
   MapDev maps[NM];
   FrameDev fr[NF];

@@ -427,31 +427,42 @@ tsdf_status read_counters(const tsdf_map* m, unsigned long long c[gbt::kNumCount
   return TSDF_OK;
 }
 
+// Scratch of the meshing and the ESDF layer: whatever of it was allocated.
+// The layer is off afterwards, and its first call allocates it again.
+void free_mesh(tsdf_map* m) {
+  cudaFree(m->mesh.list);
+  cudaFree(m->mesh.stamp);
+  cudaFree(m->mesh.cnt);
+  cudaFreeHost(m->mesh.host);
+  std::memset(&m->mesh, 0, sizeof(m->mesh));
+  m->mesh_on = false;
+}
+
+void free_esdf(tsdf_map* m) {
+  cudaFree(m->esdf.st);
+  cudaFree(m->esdf.st2);
+  cudaFree(m->esdf.list);
+  cudaFree(m->esdf.tlist[0]);
+  cudaFree(m->esdf.tlist[1]);
+  cudaFree(m->esdf.nbr);
+  cudaFree(m->esdf.clist);
+  cudaFree(m->esdf.stamp_s);
+  cudaFree(m->esdf.stamp_t);
+  cudaFree(m->esdf.ver);
+  cudaFree(m->esdf.bits);
+  cudaFree(m->esdf.cnt);
+  cudaFree(m->esdf.stats);
+  cudaFreeHost(m->esdf_host);
+  std::memset(&m->esdf, 0, sizeof(m->esdf));
+  m->esdf_host = nullptr;
+  m->esdf_on = false;
+}
+
 void free_map(tsdf_map* m) {
   cudaFree(m->more_base);
   cudaFree(m->dev.dirty);
-  if (m->mesh_on) {
-    cudaFree(m->mesh.list);
-    cudaFree(m->mesh.stamp);
-    cudaFree(m->mesh.cnt);
-    cudaFreeHost(m->mesh.host);
-  }
-  if (m->esdf_on) {
-    cudaFree(m->esdf.st);
-    cudaFree(m->esdf.st2);
-    cudaFree(m->esdf.list);
-    cudaFree(m->esdf.tlist[0]);
-    cudaFree(m->esdf.tlist[1]);
-    cudaFree(m->esdf.nbr);
-    cudaFree(m->esdf.clist);
-    cudaFree(m->esdf.stamp_s);
-    cudaFree(m->esdf.stamp_t);
-    cudaFree(m->esdf.ver);
-    cudaFree(m->esdf.bits);
-    cudaFree(m->esdf.cnt);
-    cudaFree(m->esdf.stats);
-    cudaFreeHost(m->esdf_host);
-  }
+  free_mesh(m);
+  free_esdf(m);
   if (m->aux) cudaStreamDestroy(m->aux);
   if (m->copy) cudaStreamDestroy(m->copy);
   for (int i = 0; i < 4; ++i)
@@ -1142,8 +1153,11 @@ tsdf_status esdf_alloc(tsdf_map* m, const tsdf_esdf_opts& o) {
          cudaMemset(e.ver, 0, sizeof(uint32_t) * nb) == cudaSuccess &&
          cudaMemset(e.stats, 0, sizeof(unsigned long long) * 4) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;
-  m->esdf_on = true;  // free_map releases whatever was allocated
-  if (!ok) return cuda_fail();
+  if (!ok) {  // the layer stays off: nothing may use a part of it
+    free_esdf(m);
+    return cuda_fail();
+  }
+  m->esdf_on = true;
   e.site_eps = o.site_eps;
   e.min_weight = o.min_weight;
   e.max_dist = o.max_dist_vox;
@@ -1370,13 +1384,15 @@ tsdf_status map_mesh(tsdf_map* map, float min_weight, int32_t changed_only, floa
   gbt::MeshDev& md = map->mesh;
   if (!map->mesh_on) {
     std::memset(&md, 0, sizeof(md));
-    map->mesh_on = true;  // free_map releases whatever was allocated
     if (cudaMalloc(&md.list, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
         cudaMalloc(&md.stamp, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
         cudaMalloc(&md.cnt, sizeof(unsigned long long) * 2) != cudaSuccess ||
         cudaMallocHost(&md.host, sizeof(unsigned long long) * 2) != cudaSuccess ||
-        cudaMemset(md.stamp, 0, sizeof(uint32_t) * map->max_blocks) != cudaSuccess)
+        cudaMemset(md.stamp, 0, sizeof(uint32_t) * map->max_blocks) != cudaSuccess) {
+      free_mesh(map);  // nothing may use a part of it
       return cuda_fail();
+    }
+    map->mesh_on = true;
     map->mesh_gen = 0;
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;

@@ -1388,7 +1388,8 @@ tsdf_status map_mesh(tsdf_map* map, float min_weight, int32_t changed_only, floa
         cudaMalloc(&md.stamp, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
         cudaMalloc(&md.cnt, sizeof(unsigned long long) * 2) != cudaSuccess ||
         cudaMallocHost(&md.host, sizeof(unsigned long long) * 2) != cudaSuccess ||
-        cudaMemset(md.stamp, 0, sizeof(uint32_t) * map->max_blocks) != cudaSuccess) {
+        cudaMemset(md.stamp, 0, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
+        cudaDeviceSynchronize() != cudaSuccess) {  // the caller's stream may not wait for the default one
       free_mesh(map);  // nothing may use a part of it
       return cuda_fail();
     }

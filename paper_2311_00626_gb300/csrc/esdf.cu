@@ -792,9 +792,12 @@ cudaError_t launch_esdf_reset(const MapDev& m, const EsdfDev& e, cudaStream_t s)
 }
 
 // The lowering iterations, launched cooperatively with every CTA that can be
-// resident.  Exchange generations start at gen.  The neighbour table is built
-// here unless the mark stage of an occupancy layer built it.  wait_extra: the
-// barriers' test hook.
+// resident.  A stream may have fewer SMs than the device (an MPS share, a
+// green context): a launch that is refused as too large is made with half the
+// CTAs, down to one, which meets only itself at the barriers and needs no
+// cooperative launch.  Exchange generations start at gen.  The neighbour table
+// is built here unless the mark stage of an occupancy layer built it.
+// wait_extra: the barriers' test hook.
 cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, unsigned wait_extra, cudaStream_t s) {
   static std::atomic<int> fit{0};  // resident CTAs per SM (all devices are alike here)
   int n = fit.load(std::memory_order_relaxed);
@@ -804,8 +807,8 @@ cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, u
     if (n <= 0) return cudaErrorNotSupported;
     fit.store(n, std::memory_order_relaxed);
   }
+  const int with_table = m.storage == kStorageOcc ? 0 : 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid_for(n));
   cfg.blockDim = dim3(kLowerThreads);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -813,7 +816,15 @@ cudaError_t launch_esdf_lower(const MapDev& m, const EsdfDev& e, uint32_t gen, u
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, esdf_lower_kernel, m, e, gen, m.storage == kStorageOcc ? 0 : 1, wait_extra);
+  for (int ctas = grid_for(n); ctas > 1; ctas /= 2) {
+    cfg.gridDim = dim3(ctas);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, esdf_lower_kernel, m, e, gen, with_table, wait_extra);
+    if (err != cudaErrorCooperativeLaunchTooLarge && err != cudaErrorNotSupported) return err;
+    cudaGetLastError();
+  }
+  cfg.gridDim = dim3(1);
+  cfg.numAttrs = 0;
+  return cudaLaunchKernelEx(&cfg, esdf_lower_kernel, m, e, gen, with_table, wait_extra);
 }
 
 cudaError_t launch_esdf_query(const MapDev& m, const EsdfDev& e, const float* pts, int64_t n,

@@ -283,7 +283,10 @@ tsdf_status lidar_table(tsdf_map* m, const tsdf_lidar* c, const float** out, int
   }
   LidarTable t{c->n_az, c->n_el, c->theta_start, c->phi_start, c->el_fov, nullptr, low};
   if (cudaMalloc(&t.dev, h.size() * sizeof(float)) != cudaSuccess) return cuda_fail();
-  if (cudaMemcpy(t.dev, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) {
+  // the copy of pageable memory may end after the call, and the caller's
+  // stream may not wait for the default one
+  if (cudaMemcpy(t.dev, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaStreamSynchronize(nullptr) != cudaSuccess) {
     cudaFree(t.dev);
     return cuda_fail();
   }

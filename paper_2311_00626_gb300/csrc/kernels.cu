@@ -28,6 +28,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cfloat>
+#include <cmath>
 
 #include "tsdf_internal.cuh"
 
@@ -1855,6 +1856,30 @@ cudaError_t launch_k(void (*k)(P), dim3 g, dim3 b, cudaStream_t s, const P& p) {
 // about 20 us: one 640x480 frame 22 us against 12 us by rows, eight frames 28
 // against 32, 32 frames 48 against 99, 24 frames of 1280x720 at 5 cm voxels
 // 61 against 184; the lines cross near kPatchPixels.
+//
+// And where a patch's pixels mostly share their blocks: `span` is the pixels
+// that a voxel covers at one metre, |f| v.  Below 5 the test fails nearly
+// everywhere at room distances, and below 1 cm a tile's window (32 blocks,
+// 2.6 m) does not hold a room's depths either, so that only large images or
+// launches gain (us, rows against patches; 32 frames of 640x480 unless said):
+//   1 cm     107 /  86     320x240 at 1.25 cm  45 /  55     at 1 cm  44 / 64
+//   7.5 mm   118 / 141     1280x720 x 16      145 / 118
+//   5 mm     131 / 213     1280x720 x 16      155 / 196
+//                          1920x1080 x 8      161 / 150     one      32 / 60
+//                          3840x2160 x 2      154 / 120     one      81 / 78
+//   3 mm                   3840x2160 x 2      163 / 156     one      88 / 101
+// Scenes deeper than a room at fine voxels still lose (2 cm, an open lot to 20
+// m: 96 / 130): the host does not see depths.
+constexpr float kFineVoxel = 0.0099f;   // m
+constexpr float kPatchSpan = 5.0f;      // least span of voxels from kFineVoxel up,
+constexpr float kFineSpan = 15.0f;      // of finer ones,
+constexpr float kFineSpanLarge = 7.5f;  // of finer ones in launches of kFinePixels or more
+constexpr int64_t kFinePixels = 10000000;
+inline bool patches_share_blocks(float span, float v, int64_t pixels) {
+  if (v >= kFineVoxel) return span >= kPatchSpan;
+  return span >= (pixels >= kFinePixels ? kFineSpanLarge : kFineSpan);
+}
+
 template <int NF, int NM>
 AllocShape pick_alloc_shape(const BatchParams<NF, NM>& p, int tile_h) {
   bool pinhole = false, ok = true;
@@ -1867,8 +1892,13 @@ AllocShape pick_alloc_shape(const BatchParams<NF, NM>& p, int tile_h) {
     pixels += (int64_t)F.width * F.height;
     tiny_tiles += (int64_t)((F.width + kTileW - 1) / kTileW) * ((F.height + kTileHTiny - 1) / kTileHTiny);
   }
-  if (ok && pinhole && (tile_h ? tile_h == kTileHBig : pixels >= kPatchPixels))
-    return AllocShape{kPatchTile, kTileHTiny};
+  bool patches = ok && pinhole && (tile_h ? tile_h == kTileHBig : pixels >= kPatchPixels);
+  for (int f = 0; patches && !tile_h && f < p.n_frames; ++f) {
+    const FrameDev& F = p.fr[f];
+    const float v = p.maps[NM == 1 ? 0 : F.map].v;
+    if (F.kind == kSensorPinhole) patches = patches_share_blocks(std::min(std::fabs(F.fu), std::fabs(F.fv)) * v, v, pixels);
+  }
+  if (patches) return AllocShape{kPatchTile, kTileHTiny};
   const bool big = tile_h ? tile_h == kTileHBig : pixels >= kBigTilePixels;
   // Tiles of 8 rows walk one pixel per thread instead of two: less latency
   // where they still fit one wave (a 64x48 call 16.5 -> 14.5 us, 640x480
@@ -1900,8 +1930,8 @@ cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, AllocSha
     return ph ? launch_k(band_alloc_kernel<NF, NM, kTileHTiny, true, false, true, false>, g, b, s, p)
               : launch_k(band_alloc_kernel<NF, NM, kTileHTiny, false, false, true, false>, g, b, s, p);
   if (big) {
-    // pinhole batches of this size with fast reciprocals take patch tiles
-    if (ph) return launch_k(band_alloc_kernel<NF, NM, kTileHBig, true, false, false, false>, g, b, s, p);
+    if (ph) return fast ? launch_k(band_alloc_kernel<NF, NM, kTileHBig, true, false, true, false>, g, b, s, p)
+                        : launch_k(band_alloc_kernel<NF, NM, kTileHBig, true, false, false, false>, g, b, s, p);
     return fast ? launch_k(band_alloc_kernel<NF, NM, kTileHBig, false, false, true, false>, g, b, s, p)
                 : launch_k(band_alloc_kernel<NF, NM, kTileHBig, false, false, false, false>, g, b, s, p);
   }

@@ -88,8 +88,26 @@ def test_surfaces_on_both_sides_of_the_window(voxel):
     _compare(frames, voxel, 32)
 
 
-def test_a_large_frame_takes_patches_by_itself():
-    w, h = 1600, 1000  # above the 3 << 19 pixels of the rule
+@pytest.mark.parametrize("w,h,f,voxel,n,patches", [
+    (1600, 1000, 1280.0, 0.05, 1, True),     # above the 3 << 19 pixels of the rule
+    (640, 480, 525.0, 0.05, 4, False),       # below
+    (640, 480, 525.0, 0.01, 8, True),        # a voxel spans 5.25 pixels at 1 m
+    (640, 480, 470.0, 0.01, 8, False),       # 4.7
+    (1600, 1000, 1280.0, 0.009, 1, False),   # finer than 1 cm: 11.5 of 15
+    (1600, 1000, -1280.0, 0.009, 7, True),   # 11.5 of 7.5 in a launch of 11 M pixels
+    (1600, 1000, 1700.0, 0.009, 1, True),    # 15.3
+])
+def test_which_launches_take_patches(w, h, f, voxel, n, patches):
     j, i = np.mgrid[0:h, 0:w]
-    d = (2.0 + 0.5 * np.sin(i / 90.0) + 0.3 * np.cos(j / 70.0)).astype(np.float32)
-    _compare([(_camera(w, h), np.eye(4), torch.from_numpy(d).cuda())], 0.05, 0, batch=False)
+    d = torch.from_numpy((1.0 + 0.2 * np.sin(i / 90.0) + 0.1 * np.cos(j / 70.0)).astype(np.float32)).cuda()
+    T = np.eye(4)
+    frames = []
+    for k in range(n):
+        T[0, 3] = 0.01 * k
+        frames.append((_camera(w, h, f), T.copy(), d))
+    names, got = _kernels(lambda: _run(frames, voxel, 0, False, n > 1))
+    assert ("patch_alloc_kernel" in names) == patches
+    want = _run(frames, voxel, 0, True, n > 1)
+    assert got[1:] == want[1:]
+    for a, b in zip(got[0], want[0]):
+        np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))

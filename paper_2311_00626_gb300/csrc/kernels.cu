@@ -1950,8 +1950,13 @@ cudaError_t launch_band_alloc(const BatchParams<NF, NM>& p, int n_ctas, AllocSha
 // SM: 56.6, 55.1, 55.3, 61.8, 61.4); a single frame's launch leaves room for the
 // next call's allocation, which starts while it drains (eight 640x480 calls,
 // us in all with 3, 4, 5, 6, 7: 126.5, 120.1, 120.4, 123.8, 125.5).  LiDAR scans
-// want every warp (four scans with 4, 5, 6, 7: 271, 252, 242, 231 us).
+// want every warp (four scans with 4, 5, 6, 7: 271, 252, 242, 231 us), and so do
+// maps of fine voxels, whose lists are ten thousand entries and more (with 5 and
+// 7, us: 32 frames of 640x480 at 1.25 cm 109 and 109, at 1 cm 147 and 143, at 5
+// mm 686 and 650; one 1920x1080 frame at 1.25 cm 18 and 18, at 1 cm 22 and 19, at 5
+// mm 75 and 61).
 constexpr int kPinholePerSm = 5;
+constexpr float kLimitVoxel = 0.011f;  // least voxel edge with the limit, m
 template <class P>
 cudaError_t launch_persistent(void (*k)(P), int per_sm, int limit, cudaStream_t s, const P& p,
                               std::atomic<int>& fit) {
@@ -1990,7 +1995,9 @@ cudaError_t launch_integrate(const BatchParams<NF, NM>& p, int per_sm, cudaStrea
   for (int k = 0; k < p.n_maps; ++k) wt = wt || p.maps[k].weighting != 0;
   // FAST: pinhole reciprocals by rcp_dec<true> (the host checked their range)
   const bool fast = p.fast_rcp != 0;
-  const int limit = ph && st != kStorageColor ? kPinholePerSm : 0;
+  float v = p.maps[0].v;
+  for (int k = 1; k < p.n_maps; ++k) v = std::min(v, p.maps[k].v);
+  const int limit = ph && st != kStorageColor && v >= kLimitVoxel ? kPinholePerSm : 0;
 #define GBT_INTEG(ST, PH) \
   (fast ? launch_variant<NF, NM, ST, PH, false, true>(p, per_sm, limit, s) \
         : launch_variant<NF, NM, ST, PH, false, false>(p, per_sm, limit, s))

@@ -1145,12 +1145,14 @@ __device__ __forceinline__ float2 neg_rcp2(float2 z) {
 constexpr float kFloorMagic = 12582912.0f;
 constexpr uint32_t kFloorBits = 0x4B400000u;
 
-// The constant-weight TSDF update (apply) of a voxel pair, selected per voxel.
+// The constant-weight TSDF update (apply) of a voxel pair, selected per voxel:
+// D + (s - D) / (W + 1), rounded once after the product with the reciprocal.
+// (As the addition of a product it was contracted to this by the compiler.)
 __device__ __forceinline__ void update_pair(const MapDev& m, float* D, float* W, float2 dp, bool ok0, bool ok1) {
   const float2 wn = __fadd2_rn(make_float2(W[0], W[1]), twice(1.0f));
   const float2 D2 = make_float2(D[0], D[1]);
   const float2 diff = __ffma2_rn(D2, twice(-1.0f), make_float2(fminf(dp.x, m.tau), fminf(dp.y, m.tau)));
-  const float2 dn = __fadd2_rn(D2, __fmul2_rn(diff, make_float2(rcp_approx(wn.x), rcp_approx(wn.y))));
+  const float2 dn = __ffma2_rn(diff, make_float2(rcp_approx(wn.x), rcp_approx(wn.y)), D2);
   if (ok0) { D[0] = dn.x; W[0] = fminf(wn.x, m.wmax); }
   if (ok1) { D[1] = dn.y; W[1] = fminf(wn.y, m.wmax); }
 }
@@ -1274,8 +1276,10 @@ __device__ __forceinline__ void fuse_lidar(const FrameDev& F, const MapDev& m, c
     float2 fx[2], fy[2], d00[2], d10[2], d01[2], d11[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      // u = (theta - theta_start) alpha, rounded before 1/2 is taken off (an
-      // addition of the product could be contracted; a product with 1 is not)
+      // u = (theta - theta_start) alpha, rounded before 1/2 is taken off.  (The
+      // compiler contracts a paired addition of the product, even one written
+      // as add.rn.f32x2; this form it leaves alone, which the tests watch by
+      // comparing with the scalar form below.)
       const float2 uu = __ffma2_rn(__fmul2_rn(__fadd2_rn(th[k], twice(-F.theta_start)), twice(F.alpha)), twice(1.0f), twice(-0.5f));
       const float2 vv = __ffma2_rn(__fmul2_rn(__fadd2_rn(ph[k], twice(-F.phi_start)), twice(F.beta)), twice(1.0f), twice(-0.5f));
       const float2 tu = __fadd2_rd(uu, twice(kFloorMagic)), tv = __fadd2_rd(vv, twice(kFloorMagic));

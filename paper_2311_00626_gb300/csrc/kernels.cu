@@ -61,11 +61,9 @@ __device__ __forceinline__ float rcp_dec(float x) {
   return __fmaf_rn(y, e, y);
 }
 
-// rcp_dec of a pair: the two refinement steps on the paired FP32
+// rcp_dec<true> of a pair: the two refinement steps on the paired FP32
 // operations (per component the same round-to-nearest result).
-template <bool FAST>
 __device__ __forceinline__ float2 rcp_dec2(float a, float b) {
-  if (!FAST) return make_float2(__frcp_rn(a), __frcp_rn(b));
   float2 y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.x) : "f"(a));
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.y) : "f"(b));
@@ -840,7 +838,7 @@ __device__ __forceinline__ float2 half_tan2(float2 t) {
 // mx, mn: the larger and smaller magnitude; Y_POSITIVE: y >= 0.
 template <bool Y_POSITIVE>
 __device__ __forceinline__ float2 atan2_dec2(float2 y, float2 x, float2 mx, float2 mn) {
-  const float2 r = rcp_dec2<true>(mx.x, mx.y);
+  const float2 r = rcp_dec2(mx.x, mx.y);
   const float2 q0 = __fmul2_rn(mn, r);
   const float2 t = __ffma2_rn(__ffma2_rn(make_float2(-mx.x, -mx.y), q0, mn), r, q0);
   const float2 t2 = half_tan2(half_tan2(t));

@@ -833,8 +833,8 @@ __device__ __forceinline__ float2 half_tan2(float2 t) {
 
 // atan2_dec of two voxels whose larger magnitude is in [2^-30, 2^31] and whose
 // smaller one is 0 or at least 2^-80: the quotient mn / mx by the correctly
-// rounded reciprocal and one residual step (Markstein's theorem; nothing
-// underflows in this range).
+// rounded reciprocal and one residual step (as div_voxel; nothing underflows
+// in this range).
 // mx, mn: the larger and smaller magnitude; Y_POSITIVE: y >= 0.
 template <bool Y_POSITIVE>
 __device__ __forceinline__ float2 atan2_dec2(float2 y, float2 x, float2 mx, float2 mn) {

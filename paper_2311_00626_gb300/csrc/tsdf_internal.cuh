@@ -269,10 +269,10 @@ constexpr int kPointsPerThread = 4;
 
 // Quotients of the points by the voxel edge, rounded to nearest as x / v is:
 // by the correctly rounded reciprocal and one residual step (Markstein's
-// method; equal to the division on the 93 M quotients that lie within 31 parts
-// of 2^25 units of a rounding boundary, for every odd divisor significand)
-// where nothing underflows, else by division.  inv_v = 0 selects division (set
-// by the host for extreme voxel edges).
+// method; equal to the division on the 93 M quotients that lie closest to a
+// rounding boundary, within 31 / 2^24 of a last place, for every odd divisor
+// significand) where nothing underflows, else by division.  inv_v = 0 selects
+// division (set by the host for extreme voxel edges).
 __device__ __forceinline__ float div_voxel(float x, float v, float inv_v) {
   if (fabsf(x) < 0x1p-60f || inv_v == 0.0f) return __fdiv_rn(x, v);
   const float q = __fmul_rn(x, inv_v);

@@ -454,9 +454,9 @@ constexpr int kPatchesX = kPatchTile / 4;
 static_assert(kPatchesX * kPatchesX == kAllocThreads, "one thread per patch");
 
 struct PatchSmem {
-  uint32_t bm[kWin * kWin];             // bit x of word y + 32 z: the block is in the tile's set
+  __align__(16) uint32_t bm[kWin * kWin];  // bit x of word y + 32 z: the block is in the tile's set
   uint32_t keys[kPatchKeys];            // the set's keys in order of insertion
-  uint32_t out[1 << kOutBits];          // claimed keys outside the window (claimed_outside)
+  __align__(8) uint32_t out[1 << kOutBits];  // claimed keys outside the window (claimed_outside)
   __align__(16) float4 row[kPatchTile]; // fma(M[3k+1], ry, M[3k+2]) per pixel row
   float rx[kPatchTile];                 // (i - cu) / fu per pixel column
   uint32_t nkeys, lo;                   // lo, hi: the tile's depth range (depth_range)
@@ -584,8 +584,9 @@ __device__ __forceinline__ void patch_tile(const BatchParams<NF, NM>& p, const F
   const int tiles_x = (F.width + kPatchTile - 1) / kPatchTile;
   const int x0 = (tile % tiles_x) * kPatchTile, y0 = (tile / tiles_x) * kPatchTile;
   const int px = (t % kPatchesX) * 4, py = (t / kPatchesX) * 4;  // this thread's patch in the tile
-  for (int i = t; i < kWin * kWin; i += NT) sm.bm[i] = 0u;
-  for (int i = t; i < 1 << kOutBits; i += NT) sm.out[i] = kEmptyRel;
+  static_assert(kWin * kWin == 4 * NT && (1 << kOutBits) == 2 * NT, "one store each per thread");
+  reinterpret_cast<uint4*>(sm.bm)[t] = make_uint4(0u, 0u, 0u, 0u);
+  reinterpret_cast<uint2*>(sm.out)[t] = make_uint2(kEmptyRel, kEmptyRel);
   for (int i = t; i < 2 * kPatchTile; i += NT) {
     if (i < kPatchTile) {
       sm.rx[i] = __fdiv_rn(__fsub_rn((float)(x0 + i), F.cu), F.fu);

@@ -1384,6 +1384,7 @@ tsdf_status map_mesh(tsdf_map* map, float min_weight, int32_t changed_only, floa
       map->storage != TSDF_STORAGE_FIXED16)
     return TSDF_ERR_ARG;
   if (!on_device(map)) return TSDF_ERR_STATE;
+  cudaStream_t s = (cudaStream_t)cuda_stream;
   gbt::MeshDev& md = map->mesh;
   if (!map->mesh_on) {
     std::memset(&md, 0, sizeof(md));
@@ -1391,15 +1392,14 @@ tsdf_status map_mesh(tsdf_map* map, float min_weight, int32_t changed_only, floa
         cudaMalloc(&md.stamp, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
         cudaMalloc(&md.cnt, sizeof(unsigned long long) * 2) != cudaSuccess ||
         cudaMallocHost(&md.host, sizeof(unsigned long long) * 2) != cudaSuccess ||
-        cudaMemset(md.stamp, 0, sizeof(uint32_t) * map->max_blocks) != cudaSuccess ||
-        cudaDeviceSynchronize() != cudaSuccess) {  // the caller's stream may not wait for the default one
+        // on the caller's stream, which may not wait for the default one
+        cudaMemsetAsync(md.stamp, 0, sizeof(uint32_t) * map->max_blocks, s) != cudaSuccess) {
       free_mesh(map);  // nothing may use a part of it
       return cuda_fail();
     }
     map->mesh_on = true;
     map->mesh_gen = 0;
   }
-  cudaStream_t s = (cudaStream_t)cuda_stream;
   if (cudaMemsetAsync(md.cnt, 0, sizeof(unsigned long long) * 2, s) != cudaSuccess ||
       gbt::launch_mesh(map->dev, md, mesh_table(), changed_only ? 1 : 0, ++map->mesh_gen, min_weight,
                        tri_pos_dev, tri_keys_dev, tri_cube_dev, cap, s) != cudaSuccess ||
